@@ -71,6 +71,8 @@ def draw(rng):
         while op == "fit" and case["p"] * math.prod(n) * P * P > 3e10:  # the listed fit's Gram matrix
             n = case["n"] = [max(24, v * 4 // 5) for v in n]
             case["p"] = max(1, case["p"] - 1)
+        if op == "fit" and case["p"] % 2 and all(v % 2 for v in n):
+            case["p"] += 1  # 64-bit transforms of an odd number of values are not accepted
         return dict(case, n="x".join(map(str, n)))
     snap = rng.choice(SNAPS)
     pad = rng.randint(8, 24)
