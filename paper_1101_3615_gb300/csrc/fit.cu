@@ -16,15 +16,15 @@
 // accuracy of a Householder QR (error ~ cond(A) eps) instead of the
 // cond(A)^2 eps of the normal equations M c = A^T y that Sec. 1.4 writes; the
 // first Cholesky factorisation fails (PROBE_ERR_STATE) only when A is
-// numerically rank deficient.  Gram matrices: P <= 64 -- columns formed on the
-// fly in shared memory, 32 rows at a time (pass 2 applies R1^{-1} to the staged
-// rows in shared memory); P up to 1024 -- [A | y] formed in column-major chunks
+// numerically rank deficient.  Gram matrices: P <= 64 -- pass 1 from the sums over the trials at each
+// point (k_fit_gram_s), pass 2 with the columns formed and solved against R1 in shared memory, one row
+// per thread (k_fit_gram<true>); P up to 1024 -- [A | y] formed in column-major chunks
 // of about 256 MB, R1^{-1} applied row by row, and a tiled FP64 Gram kernel.
 // A second pass forms ||y - sum_i c_i B_i x|| / ||y||.
 //
-// probe_apply_precond (end of Sec. 1.5): one D2Z transform of the image, one
-// combined multiplier gamma_lam(k) = sum_m c_(lam,m) beta_m(k) per spatial mode,
-// a batched Z2D transform, and out = sum_lam alpha_lam * w_lam.
+// probe_apply_precond (end of Sec. 1.5): one D2Z transform of the image, the spectrum times the
+// combined multiplier sum_m c_(lam,m) beta_m(k) of each spatial mode (k_precond_spectra), a batched
+// Z2D transform, and out = sum_lam alpha_lam * w_lam.
 //
 // cuFFT provides the plain FFTs; every other step is a kernel of this file.
 #include <cufft.h>
@@ -49,6 +49,8 @@ constexpr int kMaxRadial = 16;
 constexpr int kMaxMult = 32;      // nangular * nradial
 constexpr int kGramRows = 32;     // rows staged per Gram iteration
 constexpr int kGramBlocks = 608;  // 4 CTAs per SM
+constexpr int kGqBlocks = 304;    // 2 CTAs of 128 staged rows (100 KB) per SM
+constexpr size_t kGramSmemMax = 100 << 10;  // staged factors of k_fit_gram_s: at least 2 CTAs per SM
 constexpr long long kChunkBytes = 256ll << 20;  // large-P path: [A | y] chunk size
 
 struct BasisDev {
@@ -109,50 +111,135 @@ __global__ void k_fit_pad(const float* __restrict__ src, double* __restrict__ ds
     }
 }
 
-// beta_m(k) for every multiplier m = a * nradial + q on the half (real-FFT) grid
-__global__ void k_fit_beta(double* __restrict__ beta, BasisDev B) {
-    const long long tot = (long long)B.NM * B.Ncplx;
+// The k-space factors of one bin of the half (real-FFT) grid: t, the argument of the Chebyshev
+// polynomials, |k|^order (0 on the bins that every term maps to zero) and the unit wave vector.
+struct KBin {
+    double t, kpow, uz, uy, ux;
+};
+
+__device__ __forceinline__ KBin kbin(const BasisDev& B, long long r) {
     const int hx = B.Nf[2] / 2 + 1;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
+    const int jx = (int)(r % hx);
+    r /= hx;
+    const int jy = (int)(r % B.Nf[1]);
+    const int jz = (int)(r / B.Nf[1]);
+    auto freq = [](int j, int N) { return (j <= (N - 1) / 2) ? j : j - N; };
+    const double two_pi = 6.283185307179586476925286766559;
+    const double kz = two_pi * freq(jz, B.Nf[0]) / (B.Nf[0] * B.h[0]);
+    const double ky = (B.ndim == 3) ? two_pi * freq(jy, B.Nf[1]) / (B.Nf[1] * B.h[1]) : 0.0;
+    const double kx = two_pi * jx / (B.Nf[2] * B.h[2]);
+    bool nyq = ((B.Nf[0] % 2) == 0 && jz == B.Nf[0] / 2) || ((B.Nf[2] % 2) == 0 && jx == B.Nf[2] / 2);
+    if (B.ndim == 3) nyq = nyq || ((B.Nf[1] % 2) == 0 && jy == B.Nf[1] / 2);
+    const double kn = sqrt(kz * kz + ky * ky + kx * kx);
+    KBin k = {0.0, 0.0, 0.0, 0.0, 0.0};
+    if (kn > 0.0 && !nyq) {
+        const double inv = 1.0 / kn;
+        k.uz = kz * inv;
+        k.uy = ky * inv;
+        k.ux = kx * inv;
+        k.t = (kn - B.L) / (kn + B.L);
+        k.kpow = (B.order == -1.0) ? inv : (B.order == 0.0 ? 1.0 : pow(kn, B.order));
+    }
+    return k;
+}
+
+// Angular factor.  2D: cos(q theta), sin(|q| theta) with e^{i theta} = ux + i uz, as the |q|-th
+// power of that unit number by repeated squaring (no inverse or direct trigonometric function).
+__device__ __forceinline__ double angular_factor(const BasisDev& B, const KBin& k, int ang) {
+    if (B.ndim == 2) {
+        double c = 1.0, s = 0.0, bc = k.ux, bs = k.uz;
+        for (int e = abs(ang); e; e >>= 1) {
+            if (e & 1) {
+                const double t = c * bc - s * bs;
+                s = c * bs + s * bc;
+                c = t;
+            }
+            const double t = bc * bc - bs * bs;
+            bs = 2.0 * bc * bs;
+            bc = t;
+        }
+        return ang >= 0 ? c : s;
+    }
+    switch (ang) {
+        case 0: return 1.0;
+        case 1: return k.ux * k.uy;
+        case 2: return k.uy * k.uz;
+        case 3: return k.ux * k.uz;
+        case 4: return k.ux * k.ux - k.uy * k.uy;
+        default: return 3.0 * k.uz * k.uz - 1.0;
+    }
+}
+
+// beta_m(k) for every multiplier m = a * nradial + q on the half (real-FFT) grid.
+// Bound by FP64 arithmetic (two FP64 lanes per SM and clock).  One thread forms all multipliers of
+// a bin: the geometry once per bin, the radial functions by the Chebyshev recurrence
+// T_{q+1} = 2 t T_q - T_{q-1}, the angular ones by products.  12 multipliers of a 160^3 transform:
+// 0.40 ms (the 200 MB written are 0.03 ms of it); cos(q acos t), atan2 and pow evaluated for every
+// multiplier took 10.4 ms.
+__global__ void k_fit_beta(double* __restrict__ beta, BasisDev B) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < B.Ncplx;
          i += (long long)gridDim.x * blockDim.x) {
-        const int m = (int)(i / B.Ncplx);
-        long long r = i - (long long)m * B.Ncplx;
-        const int jx = (int)(r % hx);
-        r /= hx;
-        const int jy = (int)(r % B.Nf[1]);
-        const int jz = (int)(r / B.Nf[1]);
-        const int a = m / B.nradial, q = m % B.nradial;
-        auto freq = [](int j, int N) { return (j <= (N - 1) / 2) ? j : j - N; };
-        const double two_pi = 6.283185307179586476925286766559;
-        const double kz = two_pi * freq(jz, B.Nf[0]) / (B.Nf[0] * B.h[0]);
-        const double ky = (B.ndim == 3) ? two_pi * freq(jy, B.Nf[1]) / (B.Nf[1] * B.h[1]) : 0.0;
-        const double kx = two_pi * jx / (B.Nf[2] * B.h[2]);
-        bool nyq = ((B.Nf[0] % 2) == 0 && jz == B.Nf[0] / 2) || ((B.Nf[2] % 2) == 0 && jx == B.Nf[2] / 2);
-        if (B.ndim == 3) nyq = nyq || ((B.Nf[1] % 2) == 0 && jy == B.Nf[1] / 2);
-        const double kn = sqrt(kz * kz + ky * ky + kx * kx);
-        double v = 0.0;
-        if (kn > 0.0 && !nyq) {
-            double A;
-            const int ang = B.angular[a];
-            if (B.ndim == 2) {
-                const double th = atan2(kz, kx);
-                A = (ang == 0) ? 1.0 : (ang > 0 ? cos(ang * th) : sin(-ang * th));
-            } else {
-                const double uz = kz / kn, uy = ky / kn, ux = kx / kn;
-                switch (ang) {
-                    case 0: A = 1.0; break;
-                    case 1: A = ux * uy; break;
-                    case 2: A = uy * uz; break;
-                    case 3: A = ux * uz; break;
-                    case 4: A = ux * ux - uy * uy; break;
-                    default: A = 3.0 * uz * uz - 1.0; break;
+        const KBin k = kbin(B, i);
+        for (int a = 0; a < B.nangular; ++a) {
+            const double A = angular_factor(B, k, B.angular[a]) * k.kpow;
+            double t0 = 1.0, t1 = k.t;
+            for (int q = 0; q < B.nradial; ++q) {
+                beta[(long long)(a * B.nradial + q) * B.Ncplx + i] = A * t0;
+                const double t2 = fma(2.0 * k.t, t1, -t0);
+                t0 = t1;
+                t1 = t2;
+            }
+        }
+    }
+}
+
+// Preconditioner spectra: out[lam][k] = X[k] / N * sum_m c[lam * NM + m] beta_m(k), the multipliers
+// formed in registers from the bin's geometry (no beta or gamma table in memory).  c holds the
+// coefficients with nradial padded to NQ by zeros, [lam][a][NQ].  Bound by FP64 arithmetic; one
+// pass over X and the output.  60 terms (5 modes x 12) of a 288^3 transform: 3.2 ms; with a table of
+// the 12 multipliers (58 ms), a table of the 5 combinations (1.3 ms) and a product pass, 60 ms.
+constexpr int kLamBlock = 4;  // spatial modes summed per walk over the angular factors
+template <int NQ>
+__global__ void __launch_bounds__(256) k_precond_spectra(const double2* __restrict__ X, const double* __restrict__ c,
+                                                         double2* __restrict__ out, BasisDev B, double invN) {
+    extern __shared__ double cs[];  // [nspatial rounded up to kLamBlock][nangular][NQ]
+    const int nl = (B.nspatial + kLamBlock - 1) / kLamBlock * kLamBlock;
+    for (int i = threadIdx.x; i < nl * B.nangular * NQ; i += blockDim.x) {
+        const int q = i % NQ, la = i / NQ;
+        cs[i] = (q < B.nradial && la < B.nspatial * B.nangular) ? c[la * B.nradial + q] : 0.0;
+    }
+    __syncthreads();
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < B.Ncplx;
+         i += (long long)gridDim.x * blockDim.x) {
+        const KBin k = kbin(B, i);
+        double T[NQ];
+        T[0] = 1.0;
+        if (NQ > 1) T[1] = k.t;
+#pragma unroll
+        for (int q = 2; q < NQ; ++q) T[q] = fma(2.0 * k.t, T[q - 1], -T[q - 2]);
+        const double sc = k.kpow * invN;
+        const double2 x = X[i];
+        for (int l0 = 0; l0 < B.nspatial; l0 += kLamBlock) {
+            double g[kLamBlock] = {0.0, 0.0, 0.0, 0.0};
+            for (int a = 0; a < B.nangular; ++a) {
+                const double A = angular_factor(B, k, B.angular[a]);
+#pragma unroll
+                for (int l = 0; l < kLamBlock; ++l) {
+                    if (l0 + l >= B.nspatial) break;
+                    const double* cl = cs + ((l0 + l) * B.nangular + a) * NQ;
+                    double s = cl[0];
+#pragma unroll
+                    for (int q = 1; q < NQ; ++q) s = fma(cl[q], T[q], s);
+                    g[l] = fma(A, s, g[l]);
                 }
             }
-            double t = (kn - B.L) / (kn + B.L);
-            t = fmin(1.0, fmax(-1.0, t));
-            v = A * cos(q * acos(t)) * pow(kn, B.order);
+#pragma unroll
+            for (int l = 0; l < kLamBlock; ++l)
+                if (l0 + l < B.nspatial) {
+                    const double v = g[l] * sc;
+                    out[(long long)(l0 + l) * B.Ncplx + i] = make_double2(v * x.x, v * x.y);
+                }
         }
-        beta[i] = v;
     }
 }
 
@@ -191,135 +278,271 @@ __global__ void k_fit_mult(const double2* __restrict__ X, const double* __restri
     }
 }
 
-// gamma_lam(k) = sum_m c[lam*NM + m] beta_m(k)
-__global__ void k_precond_gamma(const double* __restrict__ beta, const double* __restrict__ c,
-                                double* __restrict__ gamma, BasisDev B) {
-    const long long tot = (long long)B.nspatial * B.Ncplx;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int lam = (int)(i / B.Ncplx);
-        const long long k = i - (long long)lam * B.Ncplx;
-        double g = 0.0;
-        for (int m = 0; m < B.NM; ++m) g += c[lam * B.NM + m] * beta[(long long)m * B.Ncplx + k];
-        gamma[i] = g;
-    }
-}
-
 __device__ __forceinline__ double alpha_at(const double* __restrict__ alpha, int nmax, int lam, int iz, int iy, int ix) {
     const double* a = alpha + (long long)lam * 3 * nmax;
     return a[iz] * a[nmax + iy] * a[2 * nmax + ix];
 }
 
-// Small-P path (P <= 64).  Per-CTA partial sums of the upper triangle of [A y]^T [A y] (pairs
-// (i, k), i <= k <= P), the columns formed 32 rows at a time in shared memory.  QPASS (pass 2 of
-// CholeskyQR2): the staged A part of each row is first multiplied by R1^{-1} = L1^{-T} in place
-// (eight threads per row, forward substitution), so the sums are those of [Q1 y].
-template <bool QPASS>
-__global__ void __launch_bounds__(256) k_fit_gram(const double* __restrict__ w, const float* __restrict__ y,
-                                                  const double* __restrict__ alpha, int nmax, int p, BasisDev B,
-                                                  const double* __restrict__ L1, double* __restrict__ partial) {
-    const int P = B.P, PC = P + 1;
-    const int npairs = PC * (PC + 1) / 2;
-    __shared__ double cols[kGramRows][kMaxSmall + 1];
-    __shared__ double wv[kGramRows][kMaxMult];
-    __shared__ double av[kGramRows][kMaxSpatial];
-    __shared__ unsigned short pi_[(kMaxSmall + 1) * (kMaxSmall + 2) / 2], pk_[(kMaxSmall + 1) * (kMaxSmall + 2) / 2];
-    for (int t = threadIdx.x; t < npairs; t += blockDim.x) {
-        int i = 0, rem = t;
-        while (rem >= PC - i) {
-            rem -= PC - i;
-            ++i;
-        }
-        pi_[t] = (unsigned short)i;
-        pk_[t] = (unsigned short)(i + rem);
+// Small-P path (P <= 64), pass 1 of CholeskyQR2.  Column i = (lam, m) of A is alpha_lam(x) w_m(j, x),
+// so  (A^T A)_{(l,m),(l',m')} = sum_x alpha_l alpha_l' S_mm'(x),  S_mm'(x) = sum_j w_m(j,x) w_m'(j,x),
+// and (A^T y)_{(l,m)} = sum_x alpha_l sum_j w_m y.  Forming the trial sums S once per point and then
+// the (spatial pair) x (multiplier pair) sums needs about P^2/4 + p NM^2/2 multiply-adds per point
+// instead of p P^2/2.  Bound by FP64 arithmetic (two lanes per SM and clock).  128^3 points,
+// P = 60 (5 x 12), p = 4: 6.9 ms; 28.6 ms with every pair of columns summed over every row.
+// Taken with two or more spatial modes (with one, nothing is shared) and while the staged factors
+// leave two CTAs per SM.
+// "left" factors of a point: the ns (ns + 1) / 2 products alpha_l alpha_l' (l <= l'), the ns
+// alphas, and 1; "right" factors: S_mm' (m <= m'), sum_j w_m y, sum_j y^2.  Outputs: pairs x pairs,
+// then alphas x (w y), then y^2.  partial[CTA][output].
+struct GramPlan {
+    int na2, ns2, nl, nr, nout;  // pair counts, left and right factors, outputs
+};
+__host__ __device__ inline GramPlan gram_plan(const BasisDev& B) {
+    GramPlan g;
+    g.na2 = B.nspatial * (B.nspatial + 1) / 2;
+    g.ns2 = B.NM * (B.NM + 1) / 2;
+    g.nl = g.na2 + B.nspatial + 1;
+    g.nr = g.ns2 + B.NM + 1;
+    g.nout = g.na2 * g.ns2 + B.P + 1;
+    return g;
+}
+// e-th pair (a, b), a <= b < n, in row order
+__host__ __device__ inline void pair_of(int e, int n, int& a, int& b) {
+    a = 0;
+    while (e >= n - a) e -= n - a, ++a;
+    b = a + e;
+}
+constexpr int kGramOut = 7;  // outputs per thread: nout <= 7 * 256 for every P <= 64
+
+size_t gram_s_smem(const BasisDev& B) {
+    const GramPlan g = gram_plan(B);
+    return (size_t)kGramRows * (g.nl + g.nr + B.NM + 1) * 8;
+}
+
+__global__ void __launch_bounds__(256) k_fit_gram_s(const double* __restrict__ w, const float* __restrict__ y,
+                                                    const double* __restrict__ alpha, int nmax, int p, BasisDev B,
+                                                    double* __restrict__ partial) {
+    extern __shared__ double sm[];
+    const GramPlan g = gram_plan(B);
+    double* left = sm;                                   // [nl][kGramRows]
+    double* right = left + g.nl * kGramRows;             // [nr][kGramRows]
+    double* wv = right + g.nr * kGramRows;               // [NM + 1][kGramRows]: w_m(j, .), y_j
+    __shared__ long long fidx[kGramRows];
+    __shared__ unsigned char pa[kMaxSpatial * (kMaxSpatial + 1) / 2][2], pm[(kMaxMult + 1) * (kMaxMult + 2) / 2][2];
+    const int tid = threadIdx.x;
+    for (int e = tid; e < g.na2; e += 256) {
+        int a, b;
+        pair_of(e, B.nspatial, a, b);
+        pa[e][0] = (unsigned char)a, pa[e][1] = (unsigned char)b;
     }
-    constexpr int kMaxPairsPerThread = ((kMaxSmall + 1) * (kMaxSmall + 2) / 2 + 255) / 256;
-    double acc[kMaxPairsPerThread];
+    for (int e = tid; e < g.nr; e += 256) {  // right factor e: staged rows whose product it sums
+        int a, b;
+        if (e < g.ns2)
+            pair_of(e, B.NM, a, b);
+        else
+            a = (e < g.ns2 + B.NM) ? e - g.ns2 : B.NM, b = B.NM;
+        pm[e][0] = (unsigned char)a, pm[e][1] = (unsigned char)b;
+    }
+    int lo[kGramOut], ro[kGramOut];
+    double acc[kGramOut];
 #pragma unroll
-    for (int s = 0; s < kMaxPairsPerThread; ++s) acc[s] = 0.0;
-    const long long rows = (long long)p * B.npts;
-    const long long wstride = (long long)p * B.Nreal;  // between multipliers
-    const int tr = threadIdx.x >> 3, l8 = threadIdx.x & 7;  // pass 2: row and lane of the row solve
-    __syncthreads();
-    for (long long r0 = (long long)blockIdx.x * kGramRows; r0 < rows; r0 += (long long)gridDim.x * kGramRows) {
-        // stage multiplier fields, spatial modes and y for kGramRows rows
-        for (int t = threadIdx.x; t < kGramRows * (B.NM + B.nspatial + 1); t += blockDim.x) {
-            const int r = t % kGramRows, c = t / kGramRows;
-            const long long row = r0 + r;
-            double v = 0.0;
-            if (row < rows) {
-                const int j = (int)(row / B.npts);
-                const long long pt = row - (long long)j * B.npts;
-                int iz, iy, ix;
-                unravel(pt, B, iz, iy, ix);
-                if (c < B.NM)
-                    v = w[(long long)c * wstride + (long long)j * B.Nreal + fft_index(B, iz, iy, ix)];
-                else if (c < B.NM + B.nspatial)
-                    v = alpha_at(alpha, nmax, c - B.NM, iz, iy, ix);
-                else
-                    v = (double)y[row];
-            }
-            if (c < B.NM)
-                wv[r][c] = v;
-            else if (c < B.NM + B.nspatial)
-                av[r][c - B.NM] = v;
-            else
-                cols[r][P] = v;
-        }
+    for (int k = 0; k < kGramOut; ++k) {
+        const int t = tid + 256 * k;
+        int a = g.nl - 1, r = g.nr - 1;  // y^2 (also the idle slots: in bounds, not written)
+        if (t < g.na2 * g.ns2)
+            a = t / g.ns2, r = t % g.ns2;
+        else if (t < g.na2 * g.ns2 + B.P)
+            a = g.na2 + (t - g.na2 * g.ns2) / B.NM, r = g.ns2 + (t - g.na2 * g.ns2) % B.NM;
+        lo[k] = a * kGramRows;
+        ro[k] = r * kGramRows;
+        acc[k] = 0.0;
+    }
+    const long long wstride = (long long)p * B.Nreal;
+    const int lane = tid & (kGramRows - 1), grp = tid / kGramRows;
+    for (long long x0 = (long long)blockIdx.x * kGramRows; x0 < B.npts; x0 += (long long)gridDim.x * kGramRows) {
         __syncthreads();
-        for (int t = threadIdx.x; t < kGramRows * P; t += blockDim.x) {
-            const int r = t % kGramRows, i = t / kGramRows;
-            const int lam = i / B.NM, m = i % B.NM;
-            cols[r][i] = av[r][lam] * wv[r][m];
-        }
+        const bool in = x0 + lane < B.npts;
+        int iz = 0, iy = 0, ix = 0;
+        if (in) unravel(x0 + lane, B, iz, iy, ix);
+        if (grp == 0) fidx[lane] = in ? fft_index(B, iz, iy, ix) : -1;
+        for (int l = grp; l < B.nspatial; l += 256 / kGramRows)
+            left[(g.na2 + l) * kGramRows + lane] = in ? alpha_at(alpha, nmax, l, iz, iy, ix) : 0.0;
+        if (grp == 1) left[(g.nl - 1) * kGramRows + lane] = 1.0;
         __syncthreads();
-        if (QPASS) {  // q_j = (a_j - sum_{i<j} q_i L1_ji) / L1_jj for row tr, lanes l8 split the sum
-            for (int jj = 0; jj < P; ++jj) {
-                const double* Lj = L1 + (long long)jj * P;
-                double sum = 0.0;
-                for (int i = l8; i < jj; i += 8) sum = fma(cols[tr][i], Lj[i], sum);
-                sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-                sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-                sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-                if (l8 == 0) cols[tr][jj] = (cols[tr][jj] - sum) / Lj[jj];
-                __syncwarp();
+        for (int e = grp; e < g.na2; e += 256 / kGramRows)
+            left[e * kGramRows + lane] =
+                left[(g.na2 + pa[e][0]) * kGramRows + lane] * left[(g.na2 + pa[e][1]) * kGramRows + lane];
+        for (int j = 0; j < p; ++j) {
+            const long long q = fidx[lane];
+            for (int m = grp; m <= B.NM; m += 256 / kGramRows)
+                wv[m * kGramRows + lane] =
+                    q < 0 ? 0.0
+                          : (m < B.NM ? w[(long long)m * wstride + (long long)j * B.Nreal + q]
+                                      : (double)y[(long long)j * B.npts + x0 + lane]);
+            __syncthreads();
+            for (int e = grp; e < g.nr; e += 256 / kGramRows) {
+                const double v = wv[pm[e][0] * kGramRows + lane], u = wv[pm[e][1] * kGramRows + lane];
+                double* s = right + e * kGramRows + lane;
+                *s = (j == 0) ? v * u : fma(v, u, *s);
             }
             __syncthreads();
         }
+        // left and right factors of 32 points are staged: their outer product, summed.  The point
+        // index is skewed by the lane so that a warp's lanes read different banks.
 #pragma unroll
-        for (int s = 0; s < kMaxPairsPerThread; ++s) {
-            const int t = threadIdx.x + s * 256;
-            if (t < npairs) {
-                const int i = pi_[t], k = pk_[t];
-                double a = acc[s];
+        for (int k = 0; k < kGramOut; ++k) {
+            if (tid + 256 * k >= g.nout) break;
+            double a = acc[k];
 #pragma unroll 8
-                for (int r = 0; r < kGramRows; ++r) a = fma(cols[r][i], cols[r][k], a);
-                acc[s] = a;
+            for (int r = 0; r < kGramRows; ++r) {
+                const int x = (r + tid) & (kGramRows - 1);
+                a = fma(left[lo[k] + x], right[ro[k] + x], a);
             }
+            acc[k] = a;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kGramOut; ++k)
+        if (tid + 256 * k < g.nout) partial[(long long)blockIdx.x * g.nout + tid + 256 * k] = acc[k];
+}
+
+// The sum of one value over nblocks partials (stride apart) by a warp, in a fixed order.
+__device__ __forceinline__ double warp_sum_partials(const double* part, int nblocks, long long stride) {
+    double s = 0.0;
+    for (int b = threadIdx.x & 31; b < nblocks; b += 32) s += part[(long long)b * stride];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// k_fit_gram_s's outputs summed over the CTAs into the dense lower triangle of C (n x n, n = P + 1).
+__global__ void k_fit_out_to_C(const double* __restrict__ partial, int nblocks, BasisDev B, double* __restrict__ C) {
+    const GramPlan g = gram_plan(B);
+    const int n = B.P + 1;
+    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < g.nout; t += (gridDim.x * blockDim.x) >> 5) {
+        const double s = warp_sum_partials(partial + t, nblocks, g.nout);
+        if (threadIdx.x & 31) continue;
+        if (t < g.na2 * g.ns2) {
+            int l, l2, m, m2;
+            pair_of(t / g.ns2, B.nspatial, l, l2);
+            pair_of(t % g.ns2, B.NM, m, m2);
+            const int i = l * B.NM + m, k = l2 * B.NM + m2, i2 = l * B.NM + m2, k2 = l2 * B.NM + m;
+            C[(long long)max(i, k) * n + min(i, k)] = s;
+            C[(long long)max(i2, k2) * n + min(i2, k2)] = s;
+        } else {
+            C[(long long)B.P * n + (t - g.na2 * g.ns2)] = s;  // A^T y, then y^T y on the diagonal
+        }
+    }
+}
+
+// Small-P path, all column pairs over all rows: per-CTA partial sums of the upper triangle of
+// [A y]^T [A y] (pairs (i, k), i <= k <= P) or, with QPASS (pass 2 of CholeskyQR2), of [Q1 y]^T [Q1 y]
+// with Q1 = A R1^{-1} = A L1^{-T}.  Bound by FP64 arithmetic: P^2/2 multiply-adds per row for the
+// sums and as many again for the triangular solve.  A CTA stages 128 rows, one per thread; each
+// thread forms its row's columns and solves its own row (eight columns at a time in registers, the
+// factor broadcast from shared memory, the diagonal as reciprocals), so the solve needs no
+// communication; then each thread sums up to 17 pairs over the 128 rows.  Pass 1 uses this kernel
+// where the staged factors of k_fit_gram_s would not fit (few spatial modes, many multipliers).
+// Pass 2 of the fit above: 55.4 ms, 0.96 of the FP64 rate of the sums (28.6 ms) and as many
+// multiply-adds again; 149 ms when eight threads shared a row's solve through shuffles.
+constexpr int kGqRows = 128, kGqPitch = kMaxSmall + 1;
+constexpr int kGqPairs = ((kMaxSmall + 1) * (kMaxSmall + 2) / 2 + kGqRows - 1) / kGqRows;
+constexpr size_t kGqSmem = (size_t)(kGqRows * kGqPitch + kMaxSmall * kMaxSmall + kMaxSmall) * 8;
+template <bool QPASS>
+__global__ void __launch_bounds__(kGqRows) k_fit_gram(const double* __restrict__ w, const float* __restrict__ y,
+                                                      const double* __restrict__ alpha, int nmax, int p, BasisDev B,
+                                                      const double* __restrict__ L1, double* __restrict__ partial) {
+    extern __shared__ double sm[];
+    double* cols = sm;                           // [kGqRows][kGqPitch], y in column kMaxSmall
+    double* LT = cols + kGqRows * kGqPitch;      // [i][j] = L1[j][i], zero outside P x P
+    double* rinv = LT + kMaxSmall * kMaxSmall;   // 1 / L1[j][j], zero past P
+    const int P = B.P, PC = P + 1, tid = threadIdx.x;
+    const int npairs = PC * (PC + 1) / 2;
+    int ii[kGqPairs], kk[kGqPairs];
+    double acc[kGqPairs];
+#pragma unroll
+    for (int s = 0; s < kGqPairs; ++s) {
+        acc[s] = 0.0;
+        int a = 0, b = 0;
+        if (tid + s * kGqRows < npairs) pair_of(tid + s * kGqRows, PC, a, b);
+        ii[s] = (a == P) ? kMaxSmall : a;
+        kk[s] = (b == P) ? kMaxSmall : b;
+    }
+    if (QPASS) {
+        for (int t = tid; t < kMaxSmall * kMaxSmall; t += kGqRows) {
+            const int i = t / kMaxSmall, j = t % kMaxSmall;
+            LT[t] = (i < P && j < P && i <= j) ? L1[(long long)j * P + i] : 0.0;
+        }
+        if (tid < kMaxSmall) rinv[tid] = tid < P ? 1.0 / L1[(long long)tid * P + tid] : 0.0;
+    }
+    const long long rows = (long long)p * B.npts;
+    const long long wstride = (long long)p * B.Nreal;  // between multipliers
+    double* my = cols + tid * kGqPitch;
+    for (int c = P; c < kMaxSmall; ++c) my[c] = 0.0;
+    __syncthreads();
+    for (long long r0 = (long long)blockIdx.x * kGqRows; r0 < rows; r0 += (long long)gridDim.x * kGqRows) {
+        const long long row = r0 + tid;
+        if (row < rows) {
+            const int j = (int)(row / B.npts);
+            int iz, iy, ix;
+            unravel(row - (long long)j * B.npts, B, iz, iy, ix);
+            const double* wp = w + (long long)j * B.Nreal + fft_index(B, iz, iy, ix);
+            for (int l = 0; l < B.nspatial; ++l) {
+                const double al = alpha_at(alpha, nmax, l, iz, iy, ix);
+                for (int m = 0; m < B.NM; ++m) my[l * B.NM + m] = al * wp[(long long)m * wstride];
+            }
+            my[kMaxSmall] = (double)y[row];
+        } else {
+            for (int c = 0; c < P; ++c) my[c] = 0.0;
+            my[kMaxSmall] = 0.0;
+        }
+        if (QPASS) {
+            for (int jb = 0; jb < P; jb += 8) {
+                double q[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) q[c] = my[jb + c];
+                for (int i = 0; i < jb; ++i) {
+                    const double v = -my[i];
+                    const double* l = LT + i * kMaxSmall + jb;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) q[c] = fma(v, l[c], q[c]);
+                }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    q[c] *= rinv[jb + c];
+                    const double* l = LT + (jb + c) * kMaxSmall + jb;
+#pragma unroll
+                    for (int d = c + 1; d < 8; ++d) q[d] = fma(-q[c], l[d], q[d]);
+                }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) my[jb + c] = q[c];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int s = 0; s < kGqPairs; ++s) {
+            if (tid + s * kGqRows >= npairs) break;
+            const double *ci = cols + ii[s], *ck = cols + kk[s];
+            double a = acc[s];
+#pragma unroll 8
+            for (int r = 0; r < kGqRows; ++r) a = fma(ci[r * kGqPitch], ck[r * kGqPitch], a);
+            acc[s] = a;
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int s = 0; s < kMaxPairsPerThread; ++s) {
-        const int t = threadIdx.x + s * 256;
-        if (t < npairs) partial[(long long)blockIdx.x * npairs + t] = acc[s];
-    }
+    for (int s = 0; s < kGqPairs; ++s)
+        if (tid + s * kGqRows < npairs) partial[(long long)blockIdx.x * npairs + tid + s * kGqRows] = acc[s];
 }
 
-// Small-P path: the per-CTA pair sums reduced in a fixed order into the dense lower triangle of
+// k_fit_gram's per-CTA pair sums reduced in a fixed order into the dense lower triangle of
 // C (n x n, n = P + 1, row-major): C[k][i] = sum (i <= k).
 __global__ void k_fit_pairs_to_C(const double* __restrict__ partial, int nblocks, int n, double* __restrict__ C) {
     const int npairs = n * (n + 1) / 2;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < npairs; t += gridDim.x * blockDim.x) {
-        int i = 0, rem = t;
-        while (rem >= n - i) {
-            rem -= n - i;
-            ++i;
-        }
-        const int k = i + rem;
-        double s = 0.0;
-        for (int blk = 0; blk < nblocks; ++blk) s += partial[(long long)blk * npairs + t];
-        C[(long long)k * n + i] = s;
+    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < npairs; t += (gridDim.x * blockDim.x) >> 5) {
+        const double s = warp_sum_partials(partial + t, nblocks, npairs);
+        int i, k;
+        pair_of(t, n, i, k);
+        if ((threadIdx.x & 31) == 0) C[(long long)k * n + i] = s;
     }
 }
 
@@ -669,16 +892,19 @@ probe_status stage_f32(probe_t h, const float* p, size_t n, DevBuf& buf, const f
     return PROBE_OK;
 }
 
-// beta and alpha tables of a basis into the cache; returns pointers and nmax.
+// alpha tables of a basis and (beta non-null) its multiplier tables into the cache; returns pointers
+// and nmax.
 probe_status tables(probe_t h, const BasisDev& B, cudaStream_t st, double** beta, double** alpha, int* nmax) {
     FitCache& c = *h->fit;
     *nmax = std::max(B.n[0], std::max(B.n[1], B.n[2]));
-    PROBE_TRY(ensure_buf(h, c.beta, (size_t)B.NM * B.Ncplx * 8));
+    if (beta) {
+        PROBE_TRY(ensure_buf(h, c.beta, (size_t)B.NM * B.Ncplx * 8));
+        k_fit_beta<<<grid_of(B.Ncplx), 256, 0, st>>>((double*)c.beta.p, B);
+        *beta = (double*)c.beta.p;
+    }
     PROBE_TRY(ensure_buf(h, c.alpha, (size_t)B.nspatial * 3 * (*nmax) * 8));
-    k_fit_beta<<<grid_of((long long)B.NM * B.Ncplx), 256, 0, st>>>((double*)c.beta.p, B);
     k_fit_alpha<<<grid_of((long long)B.nspatial * 3 * (*nmax)), 256, 0, st>>>((double*)c.alpha.p, B, *nmax);
     PROBE_CK(h, cudaGetLastError());
-    *beta = (double*)c.beta.p;
     *alpha = (double*)c.alpha.p;
     return PROBE_OK;
 }
@@ -691,13 +917,22 @@ probe_status fit_gram(probe_t h, const BasisDev& B, const double* w, const float
     const int P = B.P, n = P + 1;
     const long long rows = (long long)p * B.npts;
     if (P <= kMaxSmall) {
+        const size_t sm = gram_s_smem(B);
+        if (!L1 && B.nspatial > 1 && sm <= kGramSmemMax) {
+            const int nout = gram_plan(B).nout;
+            PROBE_TRY(ensure_buf(h, c.part, (size_t)kGramBlocks * nout * 8));
+            PROBE_CK(h, cudaFuncSetAttribute(k_fit_gram_s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+            k_fit_gram_s<<<kGramBlocks, 256, sm, st>>>(w, yd, alpha, nmax, p, B, (double*)c.part.p);
+            k_fit_out_to_C<<<grid_of(32ll * nout), 256, 0, st>>>((const double*)c.part.p, kGramBlocks, B, C);
+            PROBE_CK(h, cudaGetLastError());
+            return PROBE_OK;
+        }
         const int npairs = n * (n + 1) / 2;
-        PROBE_TRY(ensure_buf(h, c.part, (size_t)kGramBlocks * npairs * 8));
-        if (L1)
-            k_fit_gram<true><<<kGramBlocks, 256, 0, st>>>(w, yd, alpha, nmax, p, B, L1, (double*)c.part.p);
-        else
-            k_fit_gram<false><<<kGramBlocks, 256, 0, st>>>(w, yd, alpha, nmax, p, B, nullptr, (double*)c.part.p);
-        k_fit_pairs_to_C<<<grid_of(npairs), 256, 0, st>>>((const double*)c.part.p, kGramBlocks, n, C);
+        PROBE_TRY(ensure_buf(h, c.part, (size_t)kGqBlocks * npairs * 8));
+        auto kernel = L1 ? k_fit_gram<true> : k_fit_gram<false>;
+        PROBE_CK(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGqSmem));
+        kernel<<<kGqBlocks, kGqRows, kGqSmem, st>>>(w, yd, alpha, nmax, p, B, L1, (double*)c.part.p);
+        k_fit_pairs_to_C<<<grid_of(32ll * npairs), 256, 0, st>>>((const double*)c.part.p, kGqBlocks, n, C);
         PROBE_CK(h, cudaGetLastError());
         return PROBE_OK;
     }
@@ -858,10 +1093,9 @@ extern "C" probe_status probe_apply_precond(probe_t h, const probe_basis* basis,
         if ((s = ensure_buf(h, c.Wc, (size_t)B.nspatial * B.Ncplx * 16)) != PROBE_OK) break;
         if ((s = ensure_buf(h, c.w, (size_t)B.nspatial * B.Nreal * 8)) != PROBE_OK) break;
         if ((s = ensure_buf(h, c.coef, (size_t)(2 * B.P + 8) * 8)) != PROBE_OK) break;
-        if ((s = ensure_buf(h, c.part, (size_t)B.nspatial * B.Ncplx * 8)) != PROBE_OK) break;
-        double *beta, *alpha;
+        double* alpha;
         int nmax;
-        if ((s = tables(h, B, st, &beta, &alpha, &nmax)) != PROBE_OK) break;
+        if ((s = tables(h, B, st, nullptr, &alpha, &nmax)) != PROBE_OK) break;
         cudaError_t e = cudaMemcpyAsync(c.coef.p, coeffs, (size_t)B.P * 8, cudaMemcpyDefault, st);
         if (e != cudaSuccess) { s = cuda_fail(h, e, "coefficient copy"); break; }
         cufftHandle fwd, inv;
@@ -870,10 +1104,13 @@ extern "C" probe_status probe_apply_precond(probe_t h, const probe_basis* basis,
         if ((e = cudaMemsetAsync(c.xr.p, 0, (size_t)B.Nreal * 8, st)) != cudaSuccess) { s = cuda_fail(h, e, "memset"); break; }
         k_fit_pad<<<grid_of(B.npts), 256, 0, st>>>(id, (double*)c.xr.p, 1, B);
         if ((s = fft_check(h, cufftExecD2Z(fwd, (double*)c.xr.p, (cufftDoubleComplex*)c.Xc.p), "D2Z")) != PROBE_OK) break;
-        double* gamma = (double*)c.part.p;
-        k_precond_gamma<<<grid_of((long long)B.nspatial * B.Ncplx), 256, 0, st>>>(beta, (const double*)c.coef.p, gamma, B);
-        k_fit_mult<<<grid_of((long long)B.nspatial * B.Ncplx), 256, 0, st>>>(
-            (const double2*)c.Xc.p, gamma, (double2*)c.Wc.p, B.nspatial, 1, B.Ncplx, 1.0 / (double)B.Nreal);
+        {
+            const int NQ = B.nradial <= 4 ? 4 : (B.nradial <= 8 ? 8 : 16);
+            const size_t sm = (size_t)((B.nspatial + kLamBlock - 1) / kLamBlock * kLamBlock) * B.nangular * NQ * 8;
+            auto kernel = NQ == 4 ? k_precond_spectra<4> : (NQ == 8 ? k_precond_spectra<8> : k_precond_spectra<16>);
+            kernel<<<grid_of(B.Ncplx), 256, sm, st>>>((const double2*)c.Xc.p, (const double*)c.coef.p,
+                                                     (double2*)c.Wc.p, B, 1.0 / (double)B.Nreal);
+        }
         if ((s = fft_check(h, cufftExecZ2D(inv, (cufftDoubleComplex*)c.Wc.p, (double*)c.w.p), "Z2D")) != PROBE_OK) break;
         k_precond_combine<<<grid_of(B.npts), 256, 0, st>>>((const double*)c.w.p, alpha, nmax, B, od);
         if ((e = cudaGetLastError()) != cudaSuccess) { s = cuda_fail(h, e, "precond kernels"); break; }

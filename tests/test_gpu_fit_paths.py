@@ -1,0 +1,70 @@
+"""The Gram and multiplier kernels of the fit at the edges of their ranges, against the FP64 oracle.
+
+Both routes of the first Gram pass (trial sums per point: several spatial modes; all column pairs
+per row: one mode, or too many multipliers to stage), both passes at P = 64 and below, numbers of
+points that are no multiple of the staged 32 and 128 rows, 2D and 3D, orders other than -1.
+Coefficients: 1e-6 relative to their norm, the bar of the other fit tests (condition numbers here
+stay below 1e7, so that FP64 round-off alone gives less than 1e-8).  Preconditioned images: 1e-6,
+the rounding of the FP32 output being 6e-8.
+"""
+import numpy as np
+import pytest
+
+from oracle.symbol import Basis as OBasis
+from oracle.symbol import fit as ofit
+from workloads import mini_config
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+MODES2 = [(a, b) for a in range(-3, 4) for b in range(-3, 4)]
+MODES3 = [(0, 0, 0), (1, 0, 0), (0, -1, 0), (0, 0, 1)]
+
+
+def rel(a, b):
+    a, b = np.asarray(a, np.float64), np.asarray(b, np.float64)
+    return float(np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+def setup(shape, spatial, angular, nradial, order, fft_pad):
+    from paper_1101_3615_gb300 import Basis, Probe
+    wl = mini_config(5 if len(shape) == 3 else 1, shape=shape, nt=40, ns=1, pad=4, p=1)
+    c_mean = float(np.mean(1 / np.sqrt(wl.m0.astype(np.float64))))
+    args = (spatial, angular, nradial, 2 * np.pi * 30.0 / c_mean, order, fft_pad)
+    p = Probe(wl.m0, wl.h, wl.dt, wl.nt, wl.pad, wl.src, wl.rec, wl.wavelet)
+    return wl, p, Basis(wl.ndim, *args), OBasis(wl.shape, wl.h, *args)
+
+
+@pytest.mark.parametrize("shape,spatial,angular,nradial,p", [
+    ((44, 51), MODES2[:32], [0, 2], 1, 3),             # P = 64, most spatial modes
+    ((43, 51), [(0, 0)], [0, 2, -2, 4], 2, 2),         # one mode: all pairs per row
+    ((43, 51), [(0, 0), (0, 1)], [0, 2, -2, 4, -4, 6, -6, 8], 3, 2),  # 24 multipliers, P = 48
+    ((43, 51), [(0, 0), (0, 1)], [0, 2, -2, 4, -4, 6, -6, 8, -8, 10, -10, 12, -12, 14, -14, 16], 2, 4),  # 32: per row
+    ((16, 17), MODES2[20:23], [0], 1, 1),              # fewer points than a full staging round
+    ((14, 17, 19), MODES3, [0, 4, 5, 1], 2, 2),        # 3D
+])
+def test_fit_gram_paths_match_oracle(cuda_device, shape, spatial, angular, nradial, p):
+    wl, probe, g, o = setup(shape, spatial, angular, nradial, -1.0, 5)
+    c_true = np.random.default_rng(3).standard_normal(g.P)
+    xs = np.random.default_rng(4).standard_normal((p,) + tuple(shape)).astype(np.float32)
+    ys = np.stack([o.apply(c_true, x.astype(np.float64)) for x in xs]).astype(np.float32)
+    c_orc, res_orc, cond = ofit(o, ys, xs)
+    assert cond < 1e7
+    c, res = probe.fit(g, torch.tensor(ys, device=cuda_device), torch.tensor(xs, device=cuda_device))
+    assert rel(c, c_orc) < 1e-6, cond
+    assert abs(res - res_orc) < 1e-7
+
+
+@pytest.mark.parametrize("order", [-1.0, 0.0, 0.5])
+@pytest.mark.parametrize("shape,spatial,angular,nradial", [
+    ((33, 40), MODES2[:6], [0, 2, -2, 7, -5], 5),
+    ((33, 40), [(0, 0)], [3], 1),
+    ((33, 40), MODES2[:9], [0, -4], 11),
+    ((12, 15, 16), MODES3, [0, 1, 2, 3, 4, 5], 3),
+])
+def test_precond_spectra_match_oracle(cuda_device, shape, spatial, angular, nradial, order):
+    wl, probe, g, o = setup(shape, spatial, angular, nradial, order, 3)
+    c = np.random.default_rng(8).standard_normal(g.P)
+    img = np.random.default_rng(9).standard_normal(shape).astype(np.float32)
+    got = probe.apply_precond(g, c, torch.tensor(img, device=cuda_device)).cpu().numpy()
+    assert rel(got, o.apply(c, img.astype(np.float64))) < 1e-6
