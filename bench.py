@@ -297,6 +297,9 @@ def kernel_source_hash(name):
 
 def kernel_label(pipeline, adjoint, ndim=2, cluster=False, group=1, time_block=0):
     """Kernel name and source file of the forward / adjoint step variant the handle ran."""
+    if ndim == 2 and pipeline == 1:
+        mode = "RES_ADJ" if adjoint else "RES_INC> / <RES_BORN"
+        return f"k_res2d<{mode}> (cluster-resident, one launch per field kind and checkpoint segment)", "stencil2d_res.cu"
     if ndim == 2 and time_block > 1 and not adjoint:
         return ("k_fwd2d_tb<FWD_BORN> (incident + Born fields advanced two time levels per launch)",
                 "stencil2d.cu")

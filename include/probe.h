@@ -126,9 +126,12 @@ typedef enum {
                                     adjoint.  Setting it turns that choice off. */
     PROBE_OPT_DTT_HISTORY = 8,   /* 2D: 1 = keep Dtt u^n of every step in device memory instead of
                                     checkpointing and recomputing (FP32, W (nt-1) planes); 0 (default) */
-    PROBE_OPT_AUTOTUNE = 9,      /* 1 (default): on the first call for a shape, time the 2D kernel variants
+    PROBE_OPT_AUTOTUNE = 9,      /* 1 (default): 2D grids that fit a cluster's shared memory run on the
+                                    cluster-resident kernels where those are estimated faster; otherwise, on
+                                    the first call for a shape, time the 2D kernel variants
                                     (forward and adjoint kernel, pipeline depth, rows per thread, shot group)
-                                    and keep the fastest; setting PROBE_OPT_PIPELINE, PROBE_OPT_PIPE_ROWS or
+                                    and keep the fastest; setting PROBE_OPT_TBLOCK, PROBE_OPT_TILE_Z,
+                                    PROBE_OPT_DTT_HISTORY, PROBE_OPT_PIPELINE, PROBE_OPT_PIPE_ROWS or
                                     PROBE_OPT_SHOT_GROUP turns it off */
     PROBE_OPT_PIPE_ROWS = 10,    /* 2D pipelined kernels: rows per thread R, tile 64 x 16R (1 or 2),
                                     forward and adjoint */
@@ -184,7 +187,8 @@ typedef struct {
     int shot_group;              /* shots per CTA in the adjoint */
     int tile_z;                  /* 2D tile height used */
     int ckpt_stride;             /* checkpoint spacing used */
-    int pipeline_forward;        /* 2D forward kernel: 0 one tile per CTA, 2..4 pipeline stages;
+    int pipeline_forward;        /* 2D forward kernel: 0 one tile per CTA, 1 cluster-resident (one
+                                    launch per field kind and checkpoint segment), 2..4 pipeline stages;
                                     3D: 0 one barrier per plane, 2 producer-warp refill, 3 refill by
                                     the last compute warp */
     int pipeline_adjoint;        /* 2D adjoint kernel: same encoding; 3D: as the forward, for the
@@ -193,7 +197,8 @@ typedef struct {
     int dtt_history;             /* 1 when Dtt u^n of every step was kept instead of recomputed */
     int pipeline_rows;           /* rows per thread of the pipelined forward kernels (0: not pipelined) */
     int pipeline_rows_adjoint;   /* rows per thread of the pipelined adjoint kernel */
-    int time_block;              /* 2D Born forward and recompute: time levels per launch (1 or 2) */
+    int time_block;              /* 2D Born forward and recompute: time levels per launch (1 or 2;
+                                    cluster-resident kernels: the checkpoint stride) */
     int planes_3d;               /* 3D: z planes marched by one CTA (0 for 2D) */
     int pipeline_incident;       /* 3D: as pipeline_forward, for the incident step (forward and
                                     recompute; pipeline_forward then names the Born step's) */

@@ -61,6 +61,14 @@ struct Tuned3 {
     int fam_fwd = 2, fam_inc = 2, fam_adj = 2, zc = 64;
 };
 
+// Cluster-resident 2D kernels for one workload (shots, trials, adjoint): cluster sizes of each field
+// kind; use = 0 when the one-level kernels run instead.
+struct ResSet {
+    std::vector<long long> key;  // kind, adjoint, shots, trials
+    int use = 0;
+    ResPlan inc, born, rec, adj;  // incident and Born fields of the forward; recompute and adjoint
+};
+
 struct GraphEntry {
     std::vector<long long> key;
     cudaGraphExec_t exec = nullptr;
@@ -101,6 +109,9 @@ struct probe_s {
     // receivers by pipelined-kernel tile (64 x 16R), R = 1, 2
     int* d_wrec_ptr[3] = {nullptr, nullptr, nullptr};
     int* d_wrec_idx[3] = {nullptr, nullptr, nullptr};
+    int* d_rrec_ptr = nullptr;   // 2D: receivers by grid row (CSR over Nz)
+    int* d_rrec_idx = nullptr;
+    std::vector<probe::ResSet> res_sets;
     // 2D adjoint injection: grid rows holding receivers ("bands") and the receiver cells with
     // their receivers (CSR, receiver order), built once per handle
     int* d_rrow = nullptr;       // [Nz] band index or -1

@@ -186,6 +186,49 @@ cudaError_t launch_fwd2d_pipe(FwdKind kind, int stages, const StepParams2D& p, c
 cudaError_t launch_adj2d_pipe(int nbc, bool kahan, int stages, const StepParams2D& p, int chunks, cudaStream_t st);
 size_t pipe_smem_bytes(int stages, bool adjoint, int rows);
 size_t adj2d_smem_bytes(int tile_z);
+
+// Cluster-resident 2D kernels (stencil2d_res.cu): one field per cluster, many levels per launch.
+enum ResMode { RES_INC = 0, RES_BORN = 1, RES_ADJ = 2 };
+struct ResParams2D {
+    int Nz, Nx, P, pad, nz, nx;
+    int C;               // CTAs per cluster (set by the launcher)
+    float one;           // 1, unknown to the compiler (set by the launcher)
+    int nshots, nfield;  // fields per shot (1 incident, nb Born / adjoint)
+    int n0, nsteps;      // forward: levels n0 -> n0 + nsteps; adjoint: computes mu^{n0} .. mu^{n0 - nsteps + 1}
+    int nr;
+    float cz, cx;
+    float cxm[4], czm[4];
+    float inv_dt2, vol_inv;
+    long long F;
+    float* state;        // [nshots][nfield][2][F]
+    const float* s;
+    const float* dm;     // Born: [nfield][F]
+    float* dtt;          // Dtt u^n of level n: slot slot0 + k (forward), slot0 - k (adjoint, Dtt u^{n-1}); may be null (incident)
+    long long dtt_shot_stride;
+    int slot0;
+    const float* wavelet;
+    const int* src_zx;   // [nshots][2] padded
+    const int* rec_ptr;  // receivers by grid row (CSR over Nz)
+    const int* rec_idx;
+    const int* rec_zx;   // [nr][2] padded
+    float* data;         // levels n0 .. n0 + nsteps - 1 at the receivers; may be null
+    long long dss, dts;
+    const int* rrow;     // adjoint: injection band of a grid row, -1 without receivers
+    const float* inj;    // [slots][nshots][nfield][inj_block], slot k = level n0 - k
+    long long inj_block;
+    float* img;          // adjoint: [nshots][nfield][F]
+    float* comp;
+    int* err;
+};
+struct ResPlan {
+    int C = 0, RB = 4, threads = 0;  // CTAs per cluster, rows per thread
+    int clusters = 0;                // clusters resident on the chip at once
+    double us = 0.0;                 // estimated time per level and wave of clusters
+};
+constexpr size_t kResSmemMax = 226 * 1024;  // dynamic shared memory beside the static barriers
+bool res2d_fits(int mode, bool kahan, int Nz, int Nx, int pad, int nsteps);  // in some cluster's shared memory
+std::vector<ResPlan> plan_res2d(int mode, bool kahan, int Nz, int Nx, int pad, int nsteps);
+cudaError_t launch_res2d(int mode, bool kahan, const ResPlan& pl, const ResParams2D& p, cudaStream_t st);
 cudaError_t stencil2d_configure();  // opt-in shared memory sizes
 
 // Auxiliary kernels (aux.cu).

@@ -171,20 +171,41 @@ long long inj_block(probe_t h) { return (long long)h->nband * (h->ndim == 3 ? (l
 // Bytes per resident shot and fixed bytes of a job with nb trials.
 bool use_history(probe_t h, int with_ckpt) { return with_ckpt && h->opt_dtt_history && h->ndim == 2; }
 
+// 2D calls may run on the cluster-resident kernels (stencil2d_res.cu): no kernel variant or Dtt
+// history chosen by the caller, and a strip of at least four rows of some cluster's CTA holds the
+// two levels and the pointwise operands of the fields that the call advances.
+bool res_fits(probe_t h, int with_ckpt, int born) {
+    if (h->ndim != 2 || h->user_fixed || h->user_tblock || h->opt_tile_z || h->opt_dtt_history || !h->opt_autotune)
+        return false;
+    const bool kh = h->kahan != 0;
+    return res2d_fits(RES_INC, kh, h->Nz, h->Nx, h->pad, h->K) && (!born || res2d_fits(RES_BORN, kh, h->Nz, h->Nx, h->pad, h->K)) &&
+           (!with_ckpt || res2d_fits(RES_ADJ, kh, h->Nz, h->Nx, h->pad, h->K));
+}
+
+// Dtt planes per shot of a 2D workspace: the history; two checkpoint segments for the resident
+// kernels (one being read while the next is written); one segment; none (1, unallocated).
+int dtt_slots_2d(probe_t h, int with_ckpt, int history, int res) {
+    if (history) return h->nt - 1;
+    if (res) return 2 * h->K;
+    return with_ckpt ? h->K : 1;
+}
+
 // 3D adjoint on the producer-warp kernel (receiver injection from a per-segment band buffer)
 // rather than the one-barrier-per-plane kernel or the shot-cluster kernel.
 bool adj3d_ws(probe_t h) { return h->ndim == 3 && h->pipe_adj != 0 && !(h->opt_cluster3d & 2); }
 
-void ws_bytes(probe_t h, int nb, int with_ckpt, int with_data, double* per_shot, double* fixed) {
+void ws_bytes(probe_t h, int nb, int with_ckpt, int with_data, int res, double* per_shot, double* fixed) {
     const double F4 = (double)h->F * 4.0;
     double ps = 2 * F4 + 2.0 * nb * F4;
     if (h->ndim == 2) ps += 4 * F4 + 4.0 * nb * F4;  // four-level states of the time-blocked forward
     if (use_history(h, with_ckpt))
         ps += (double)(h->nt - 1) * F4;
     else if (with_ckpt)
-        ps += (double)h->nck * ckpt_bytes_per_shot(h->snap, h->F) + (double)h->K * F4 + 16.0 * h->nck;
+        ps += (double)h->nck * ckpt_bytes_per_shot(h->snap, h->F) + (res ? 2.0 : 1.0) * h->K * F4 + 16.0 * h->nck;
     else if (h->ndim == 3)
         ps += 2.0 * F4;  // Dtt u^n of two steps (Born source)
+    else if (res)
+        ps += 2.0 * h->K * F4;
     if (with_data) ps += (double)nb * h->nt * h->nr * 4.0;
     if (h->ndim == 3 && with_ckpt) {
         ps += 2.0 * nb * F4;  // per-shot images + compensation
@@ -195,10 +216,10 @@ void ws_bytes(probe_t h, int nb, int with_ckpt, int with_data, double* per_shot,
     *fixed = nb * F4 + 2.0 * F4 * nb + F4;  // dm, one image group, s_tmp
 }
 
-int plan_wave(probe_t h, int nb, int with_ckpt, int with_data) {
+int plan_wave(probe_t h, int nb, int with_ckpt, int with_data, int res) {
     if (h->opt_shot_wave > 0) return std::min(h->opt_shot_wave, h->ns);
     double ps, fx;
-    ws_bytes(h, nb, with_ckpt, with_data, &ps, &fx);
+    ws_bytes(h, nb, with_ckpt, with_data, res, &ps, &fx);
     size_t freeb = 0, totb = 0;
     cudaMemGetInfo(&freeb, &totb);
     const double budget = 0.80 * (double)freeb + (double)h->ws.bytes;
@@ -242,11 +263,12 @@ probe_status encode_ws_maps(probe_t h, WsMaps& m, int R) {
     return PROBE_OK;
 }
 
-probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data) {
+probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, int res) {
     Workspace& w = h->ws;
     const int G = W;  // image groups for the smallest shot group: any group size fits
     const int history = use_history(h, with_ckpt) ? 1 : 0;
-    if (w.u && w.W >= W && w.nb >= nb && w.with_ckpt >= with_ckpt && w.with_data >= with_data &&
+    const int slots2 = h->ndim == 2 ? dtt_slots_2d(h, with_ckpt, history, res) : 0;
+    if (w.u && (h->ndim == 3 || w.dtt_slots == slots2) && w.W >= W && w.nb >= nb && w.with_ckpt >= with_ckpt && w.with_data >= with_data &&
         w.groups >= G && w.tm_tile_z == h->tile_z && w.W == W && w.nb == nb && w.history == history)
         return PROBE_OK;
     free_ws(w);
@@ -271,9 +293,11 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data) {
         TRY(alloc(&w.ckpt, (size_t)h->nck * W * ckpt_bytes_per_shot(h->snap, F)));
         TRY(alloc((void**)&w.scales, (size_t)h->nck * W * 2 * 4));
         TRY(alloc((void**)&w.absmax, (size_t)W * 2 * 4));
-        TRY(alloc((void**)&w.dtt, (size_t)W * h->K * F * 4));
+        TRY(alloc((void**)&w.dtt, (size_t)W * (h->ndim == 2 ? slots2 : h->K) * F * 4));
     } else if (h->ndim == 3) {
         TRY(alloc((void**)&w.dtt, (size_t)W * 2 * F * 4));  // Dtt u^n of two steps (Born source)
+    } else if (slots2 > 1) {
+        TRY(alloc((void**)&w.dtt, (size_t)W * slots2 * F * 4));
     }
     TRY(alloc((void**)&w.img, (size_t)G * std::max(nb, 1) * F * 4));
     TRY(alloc((void**)&w.comp, (size_t)G * std::max(nb, 1) * F * 4));
@@ -289,7 +313,7 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data) {
     CK(h, cudaMemset(w.u, 0, (size_t)W * 2 * F * 4));
     CK(h, cudaMemset(w.f, 0, (size_t)W * std::max(nb, 1) * 2 * F * 4));
     w.history = history;
-    w.dtt_slots = history ? h->nt - 1 : (with_ckpt ? h->K : (h->ndim == 3 ? 2 : 1));
+    w.dtt_slots = h->ndim == 2 ? slots2 : (with_ckpt ? h->K : 2);
     if (w.dtt) CK(h, cudaMemset(w.dtt, 0, (size_t)W * w.dtt_slots * F * 4));
     w.W = W;
     w.nb = nb;
@@ -400,6 +424,8 @@ probe_status build_rec_tiles(probe_t h) {
     TRY(upload_csr(h, key, nkeys, &h->d_rec_tile_ptr, &h->d_rec_tile_idx));
     if (!h->d_rrow) TRY(build_bands(h));
     if (h->ndim == 2) {
+        for (int r = 0; r < h->nr; ++r) key[r] = h->rec_pad[2 * r];  // grid rows (resident kernels)
+        TRY(upload_csr(h, key, h->Nz, &h->d_rrec_ptr, &h->d_rrec_idx));
         for (int R = 1; R <= 2; ++R) {  // tiles of the pipelined kernels (64 x 16R)
             const int tz = (h->Nz + 16 * R - 1) / (16 * R);
             for (int r = 0; r < h->nr; ++r)
@@ -826,6 +852,232 @@ probe_status run_adjoint(Sweep& sw) {
     return PROBE_OK;
 }
 
+probe_status ensure_overlap_stream(probe_t h) {
+    if (h->ostream) return PROBE_OK;
+    CK(h, cudaStreamCreateWithFlags(&h->ostream, cudaStreamNonBlocking));
+    for (int i = 0; i < 2; ++i) {
+        CK(h, cudaEventCreateWithFlags(&h->ov_inc[i], cudaEventDisableTiming));
+        CK(h, cudaEventCreateWithFlags(&h->ov_born[i], cudaEventDisableTiming));
+    }
+    return PROBE_OK;
+}
+
+// ---------------------------------------------------------------------------
+// 2D sweeps on the cluster-resident kernels: one launch per field kind and checkpoint segment.
+// ---------------------------------------------------------------------------
+void fill_res(const Job& jb, ResParams2D& p) {
+    probe_t h = jb.h;
+    Workspace& w = h->ws;
+    memset(&p, 0, sizeof(p));
+    p.Nz = h->Nz;
+    p.Nx = h->Nx;
+    p.P = h->P;
+    p.pad = h->pad;
+    p.nz = h->nz;
+    p.nx = h->nx;
+    p.nshots = jb.W;
+    p.nr = h->nr;
+    p.cz = h->cz;
+    p.cx = h->cx;
+    const double wk[4] = {PROBE_W1, PROBE_W2, PROBE_W3, PROBE_W4};
+    for (int mm = 0; mm < 4; ++mm) {
+        double cm = 0.0;
+        for (int k = mm; k < 4; ++k) cm += wk[k];
+        p.cxm[mm] = (float)(cm / (h->hx * h->hx));
+        p.czm[mm] = (float)(cm / (h->hz * h->hz));
+    }
+    p.inv_dt2 = (float)(1.0 / (h->dt * h->dt));
+    p.vol_inv = (float)(1.0 / (h->hz * h->hx));
+    p.F = h->F;
+    p.s = jb.s;
+    p.dtt_shot_stride = (long long)w.dtt_slots * h->F;
+    p.wavelet = h->d_wavelet;
+    p.src_zx = w.src_wave;
+    p.rec_ptr = h->d_rrec_ptr;
+    p.rec_idx = h->d_rrec_idx;
+    p.rec_zx = h->d_rec;
+    p.dss = jb.dss;
+    p.dts = jb.dts;
+    p.err = h->d_err;
+}
+
+// The incident field's chain (checkpoint store or restore, levels of a segment) runs on the second
+// stream, the Born / adjoint chain on the call's: segment i uses Dtt slots (i & 1) K .. + K - 1, the
+// incident launch i + 2 waits for the last reader of its slots.  Each chain alone leaves SMs idle.
+probe_status run_forward_res(Sweep& sw, Job& jb, const ResSet& rs, FwdKind kind, bool ckpt) {
+    probe_t h = jb.h;
+    Workspace& w = h->ws;
+    cudaStream_t st = sw.st;
+    const bool born = kind == FWD_BORN;
+    CK(h, cudaMemsetAsync(w.u, 0, (size_t)jb.W * 2 * h->F * 4, st));
+    if (born) CK(h, cudaMemsetAsync(w.f, 0, (size_t)jb.W * jb.nb * 2 * h->F * 4, st));
+    ResParams2D pi, pb;
+    fill_res(jb, pi);
+    pi.nfield = 1;
+    pi.state = w.u;
+    if (kind == FWD_INCIDENT_SAMPLE) pi.data = jb.data;
+    fill_res(jb, pb);
+    pb.nfield = jb.nb;
+    pb.state = w.f;
+    pb.dm = w.dm;
+    pb.dtt = w.dtt;
+    pb.data = jb.data;
+    cudaStream_t su = st;
+    if (born) {
+        TRY(ensure_overlap_stream(h));
+        su = h->ostream;
+        CK(h, cudaEventRecord(h->ov_inc[0], st));
+        CK(h, cudaStreamWaitEvent(su, h->ov_inc[0], 0));
+    }
+    for (int n = 0, i = 0; n < h->nt - 1; n += h->K, ++i) {
+        const int T = std::min(h->K, h->nt - 1 - n), set = i & 1;
+        if (born && i >= 2) CK(h, cudaStreamWaitEvent(su, h->ov_born[set], 0));
+        if (ckpt) {
+            const size_t per = (size_t)jb.W * ckpt_bytes_per_shot(h->snap, h->F);
+            cudaError_t e = launch_encode_ckpt(w.u, jb.W * 2, h->F, 2, n & 1, (n & 1) ^ 1, (char*)w.ckpt + i * per,
+                                               w.scales + (size_t)i * jb.W * 2, h->snap, w.absmax, su);
+            if (e != cudaSuccess) return cuda_fail(h, e, "checkpoint store");
+            sw.launches_other += codec_launches(h->snap, true, 2, n & 1);
+        }
+        pi.n0 = pb.n0 = n;
+        pi.nsteps = pb.nsteps = T;
+        pi.slot0 = pb.slot0 = set * h->K;
+        pi.dtt = born ? w.dtt : nullptr;
+        cudaError_t e = launch_res2d(RES_INC, false, rs.inc, pi, su);
+        if (e != cudaSuccess) return cuda_fail(h, e, "incident segment launch");
+        sw.launches_fwd++;
+        if (!born) continue;
+        CK(h, cudaEventRecord(h->ov_inc[set], su));
+        CK(h, cudaStreamWaitEvent(st, h->ov_inc[set], 0));
+        e = launch_res2d(RES_BORN, false, rs.born, pb, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "Born segment launch");
+        CK(h, cudaEventRecord(h->ov_born[set], st));
+        sw.launches_fwd++;
+    }
+    if (born || kind == FWD_INCIDENT_SAMPLE) {  // last time level at the receivers
+        cudaError_t e = launch_sample(born ? w.f : w.u, (long long)(born ? jb.nb : 1) * 2 * h->F, 2 * h->F,
+                                      (h->nt - 1) & 1, h->F, jb.W, born ? jb.nb : 1, h->d_rec, h->nr, h->P, h->ndim,
+                                      h->Ny, jb.data, jb.dss, jb.dts, h->nt - 1, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "receiver sampling");
+        sw.launches_other++;
+    }
+    return PROBE_OK;
+}
+
+probe_status run_adjoint_res(Sweep& sw, Job& jb, const ResSet& rs) {
+    probe_t h = jb.h;
+    Workspace& w = h->ws;
+    cudaStream_t st = sw.st;
+    CK(h, cudaMemsetAsync(w.f, 0, (size_t)jb.W * jb.nb * 2 * h->F * 4, st));
+    ResParams2D pi, pa;
+    fill_res(jb, pi);
+    pi.nfield = 1;
+    pi.state = w.u;
+    pi.dtt = w.dtt;
+    fill_res(jb, pa);
+    pa.nfield = jb.nb;
+    pa.state = w.f;
+    pa.dtt = w.dtt;
+    pa.rrow = h->nband > 0 ? h->d_rrow : nullptr;
+    pa.inj = w.inj;
+    pa.inj_block = inj_block(h);
+    pa.img = w.img;
+    pa.comp = w.comp;
+    TRY(ensure_overlap_stream(h));
+    cudaStream_t su = h->ostream;
+    CK(h, cudaEventRecord(h->ov_inc[0], st));
+    CK(h, cudaStreamWaitEvent(su, h->ov_inc[0], 0));
+    int ev = 2;
+    for (int k = h->nck - 1, i = 0; k >= 0; --k) {
+        const int k0 = k * h->K, k1 = std::min(k0 + h->K, h->nt - 1), set = i & 1;
+        if (k0 >= k1) continue;
+        record(h, ev++, st);
+        if (i >= 2) CK(h, cudaStreamWaitEvent(su, h->ov_born[set], 0));
+        const size_t per = (size_t)jb.W * ckpt_bytes_per_shot(h->snap, h->F);
+        cudaError_t e = launch_decode_ckpt((const char*)w.ckpt + (size_t)k * per, w.scales + (size_t)k * jb.W * 2,
+                                           jb.W * 2, h->F, 2, k0 & 1, (k0 & 1) ^ 1, h->snap, w.u, su);
+        if (e != cudaSuccess) return cuda_fail(h, e, "checkpoint restore");
+        sw.launches_other += codec_launches(h->snap, false, 2, k0 & 1);
+        pi.n0 = k0;
+        pi.nsteps = k1 - k0;
+        pi.slot0 = set * h->K;
+        e = launch_res2d(RES_INC, false, rs.rec, pi, su);
+        if (e != cudaSuccess) return cuda_fail(h, e, "recompute segment launch");
+        sw.launches_rec++;
+        CK(h, cudaEventRecord(h->ov_inc[set], su));
+        CK(h, cudaStreamWaitEvent(st, h->ov_inc[set], 0));
+        record(h, ev++, st);
+        Sweep one;  // this job's injection
+        one.jobs.push_back(jb);
+        one.st = st;
+        TRY(build_injection(one, k1, k0 + 1));
+        sw.launches_other += one.launches_other;
+        pa.n0 = k1;
+        pa.nsteps = k1 - k0;
+        pa.slot0 = set * h->K + (k1 - k0 - 1);  // level n uses Dtt u^{n-1}
+        e = launch_res2d(RES_ADJ, h->kahan != 0, rs.adj, pa, st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "adjoint segment launch");
+        CK(h, cudaEventRecord(h->ov_born[set], st));
+        sw.launches_adj++;
+        ++i;
+    }
+    record(h, ev++, st);
+    return PROBE_OK;
+}
+
+// The pair of plans for two chains of ua and ub fields that run side by side (ub = 0: one chain) with
+// the least estimated time per level.  Both chains use one cluster size: a launch of other clusters
+// beside the first leaves holes (241 x 281, 6 + 6 fields: 79 us per segment of 20 levels with clusters
+// of 8 for both, 116 us with 8 and 16).  Where both do not fit at once they run one after the other.
+double res_pair(const std::vector<ResPlan>& pa, int ua, const std::vector<ResPlan>& pb, int ub, ResPlan* a,
+                ResPlan* b) {
+    double best = 1e30;
+    auto waves = [](int u, int cl) { return (double)((u + cl - 1) / cl); };
+    for (const ResPlan& x : pa) {
+        const double tx = waves(ua, x.clusters) * x.us;
+        if (!ub && tx < best) best = tx, *a = x;
+        for (size_t i = 0; ub && i < pb.size(); ++i) {
+            const ResPlan& y = pb[i];
+            if (y.C != x.C) continue;
+            const double ty = waves(ub, y.clusters) * y.us;
+            const double t = ua + ub <= std::min(x.clusters, y.clusters) ? std::max(tx, ty) : tx + ty;
+            if (t < best) best = t, *a = x, *b = y;
+        }
+    }
+    return best;
+}
+
+// Whether a call of this kind runs on the resident kernels, with the cluster sizes (kept per
+// workload; a host-side estimate, nothing is timed).  They are taken where their estimate, with
+// 14 us per segment and chain for launch, load and store, is below the one-level kernels': one launch
+// of at least 4.5 us per level, or the rates that those reach on grids that fill the chip (360
+// Gcell/s forward, 300 recompute, 215 adjoint; 541 x 541, 32 shots).
+const ResSet& res_set(probe_t h, FwdKind kind, bool adjoint, int W, int nb) {
+    const std::vector<long long> key = {(long long)kind, (long long)adjoint, W, nb, h->user_fixed, h->user_tblock,
+                                        h->opt_tile_z, h->opt_dtt_history, h->opt_autotune};
+    for (const ResSet& r : h->res_sets)
+        if (r.key == key) return r;
+    ResSet r;
+    r.key = key;
+    const bool born = kind == FWD_BORN, kh = h->kahan != 0;
+    if (res_fits(h, adjoint, born)) {
+        const std::vector<ResPlan> inc = plan_res2d(RES_INC, kh, h->Nz, h->Nx, h->pad, h->K);
+        std::vector<ResPlan> bo, ad;
+        if (born) bo = plan_res2d(RES_BORN, kh, h->Nz, h->Nx, h->pad, h->K);
+        if (adjoint) ad = plan_res2d(RES_ADJ, kh, h->Nz, h->Nx, h->pad, h->K);
+        const double seg = 14.0 / h->K, gc = (double)h->Nz * h->Nx * W * 1e-3;  // thousand cells of one field kind
+        double t = res_pair(inc, W, bo, born ? W * nb : 0, &r.inc, &r.born) + seg;
+        double t1 = std::max(4.5, gc * (born ? 1 + nb : 1) / 360.0);
+        if (adjoint) {
+            t += res_pair(inc, W, ad, W * nb, &r.rec, &r.adj) + seg;
+            t1 += std::max(4.5, gc / 300.0) + std::max(4.5, gc * nb / 215.0);
+        }
+        r.use = t < t1;
+    }
+    h->res_sets.push_back(r);
+    return h->res_sets.back();
+}
+
 // ---------------------------------------------------------------------------
 // 3D sweeps: one launch per field kind and step (incident, Born trials, adjoint).
 // ---------------------------------------------------------------------------
@@ -1048,16 +1300,6 @@ probe_status autotune_3d(const Job& jb, FwdKind kind, bool adjoint, cudaStream_t
     t.fam_adj = h->pipe_adj;
     t.zc = h->zc3d;
     h->tuned3.push_back(t);
-    return PROBE_OK;
-}
-
-probe_status ensure_overlap_stream(probe_t h) {
-    if (h->ostream) return PROBE_OK;
-    CK(h, cudaStreamCreateWithFlags(&h->ostream, cudaStreamNonBlocking));
-    for (int i = 0; i < 2; ++i) {
-        CK(h, cudaEventCreateWithFlags(&h->ov_inc[i], cudaEventDisableTiming));
-        CK(h, cudaEventCreateWithFlags(&h->ov_born[i], cudaEventDisableTiming));
-    }
     return PROBE_OK;
 }
 
@@ -1533,7 +1775,7 @@ extern "C" void probe_destroy(probe_t h) {
     free_ws(h->ws);
     void* ptrs[] = {h->d_m0, h->d_s0, h->d_wavelet, h->d_src, h->d_rec, h->d_rec_tile_ptr, h->d_rec_tile_idx,
                     h->d_wrec_ptr[1], h->d_wrec_idx[1], h->d_wrec_ptr[2], h->d_wrec_idx[2],
-                    h->d_rrow, h->d_uc_ptr, h->d_uc_rec, h->d_uc_pos,
+                    h->d_rrec_ptr, h->d_rrec_idx, h->d_rrow, h->d_uc_ptr, h->d_uc_rec, h->d_uc_pos,
                     h->d_err, h->stage_in.p, h->stage_out.p};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -1854,9 +2096,12 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
     const bool need_ckpt = (op == OP_FADJ || op == OP_H || op == OP_GRAD);
     const bool need_data = (op == OP_H);
     const int nbw = (op == OP_NONLIN || op == OP_GRAD) ? 1 : nb;
-    const int W = plan_wave(h, nbw, need_ckpt, need_data);
-    TRY(ensure_ws(h, W, nbw, need_ckpt, need_data));
+    const FwdKind kind = (op == OP_F || op == OP_H) ? FWD_BORN : (op == OP_NONLIN) ? FWD_INCIDENT_SAMPLE : FWD_INCIDENT;
+    const int fits = res_fits(h, need_ckpt, kind == FWD_BORN);
+    const int W = plan_wave(h, nbw, need_ckpt, need_data, fits);
+    TRY(ensure_ws(h, W, nbw, need_ckpt, need_data, fits));
     Workspace& w = h->ws;
+    const ResSet rs = h->ndim == 2 ? res_set(h, kind, need_ckpt, W, nbw) : ResSet();
     int G = 0;
     reset_stats(h);
     h->stats.shot_wave = W;
@@ -1915,23 +2160,21 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
                 jb.dts = 0;
                 break;
         }
-        FwdKind kind = (op == OP_F || op == OP_H) ? FWD_BORN
-                       : (op == OP_NONLIN)        ? FWD_INCIDENT_SAMPLE
-                                                  : FWD_INCIDENT;
         if (wv == 0) {
             if (h->ndim == 2) {
                 jb.shot_group = pick_group(h, W);
                 jb.groups = (Wv + jb.shot_group - 1) / jb.shot_group;
                 const std::vector<long long> tkey = {(long long)kind, (long long)need_ckpt, Wv, nbw};
                 int grp = 0;
-                TRY(autotune_2d(h, tkey, {jb}, kind, need_ckpt, true, st, &grp));
+                if (!rs.use) TRY(autotune_2d(h, tkey, {jb}, kind, need_ckpt, true, st, &grp));
                 if (grp > 0) h->opt_shot_group = grp;
             }
-            G = (W + pick_group(h, W) - 1) / pick_group(h, W);
-            h->stats.shot_group = pick_group(h, W);
-            const bool piped = h->ndim == 2 && h->tile_z == kPipeTZ;
-            h->stats.pipeline_forward = piped ? h->opt_pipeline : 0;
-            h->stats.pipeline_adjoint = piped ? h->pipe_adj : 0;
+            const int g0 = rs.use ? 1 : pick_group(h, W);  // resident kernels: one image per shot
+            G = (W + g0 - 1) / g0;
+            h->stats.shot_group = g0;
+            const bool piped = h->ndim == 2 && h->tile_z == kPipeTZ && !rs.use;
+            h->stats.pipeline_forward = rs.use ? 1 : (piped ? h->opt_pipeline : 0);
+            h->stats.pipeline_adjoint = rs.use ? 1 : (piped ? h->pipe_adj : 0);
             if (h->ndim == 3) TRY(autotune_3d(jb, kind, need_ckpt, st));
             h->stats.planes_3d = (h->ndim == 3) ? h->zc3d : 0;
             if (h->ndim == 3) {  // 0 one barrier per plane, 2 producer warp, 3 refill by the last compute warp
@@ -1941,13 +2184,13 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
             }
             h->stats.pipeline_rows = piped ? h->ws_rows : 0;
             h->stats.pipeline_rows_adjoint = piped ? h->ws_rows_adj : 0;
-            h->stats.time_block = (h->ndim == 2 && h->tile_z == kPipeTZ && w.u4) ? h->opt_tblock : 1;
+            h->stats.time_block = rs.use ? h->K : (h->ndim == 2 && h->tile_z == kPipeTZ && w.u4) ? h->opt_tblock : 1;
             if (need_ckpt) {
                 CK(h, cudaMemsetAsync(w.img, 0, (size_t)G * nbw * h->F * 4, st));
                 CK(h, cudaMemsetAsync(w.comp, 0, (size_t)G * nbw * h->F * 4, st));
             }
         }
-        jb.shot_group = pick_group(h, W);
+        jb.shot_group = rs.use ? 1 : pick_group(h, W);
         jb.groups = (Wv + jb.shot_group - 1) / jb.shot_group;
         if (h->ndim == 3) {
             Count3 c3;
@@ -1964,16 +2207,19 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
             const std::vector<long long> key = {(long long)op, (long long)kind, (long long)need_ckpt, Wv, nbw, j0,
                                                 (long long)(size_t)jb.data, (long long)(size_t)jb.rdata,
                                                 (long long)(size_t)jb.s, h->ws.generation, h->opt_pipeline, h->pipe_adj, h->ws_rows, h->ws_rows_adj, h->opt_timing, h->opt_tblock,
-                                                jb.shot_group, h->tile_z, h->nt};
+                                                jb.shot_group, h->tile_z, h->nt, rs.use};
             long long cnt[4] = {0, 0, 0, 0};
             TRY(run_maybe_graph(h, key, st, cnt, [&](cudaStream_t ss) -> probe_status {
                 Sweep sw2;
                 sw2.jobs = sw.jobs;
-                TRY(prepare_sweep(sw2, h, ss));
+                if (rs.use)
+                    sw2.st = ss;
+                else
+                    TRY(prepare_sweep(sw2, h, ss));
                 record(h, 0, ss);
-                TRY(run_forward(sw2, kind, need_ckpt));
+                TRY(rs.use ? run_forward_res(sw2, sw2.jobs[0], rs, kind, need_ckpt) : run_forward(sw2, kind, need_ckpt));
                 record(h, 1, ss);
-                if (need_ckpt) TRY(run_adjoint(sw2));
+                if (need_ckpt) TRY(rs.use ? run_adjoint_res(sw2, sw2.jobs[0], rs) : run_adjoint(sw2));
                 cnt[0] = sw2.launches_fwd;
                 cnt[1] = sw2.launches_rec;
                 cnt[2] = sw2.launches_adj;
@@ -1999,7 +2245,9 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
         // forward (u^n, u^{n-1}, s, two writes, per trial likewise, every other level) and 14 bytes
         // for the recompute (with its two Dtt writes)
         const bool tb2 = h->ndim == 2 && h->opt_tblock == 2 && h->tile_z == kPipeTZ && w.u4;
-        if (tb2 && kind == FWD_BORN)
+        if (rs.use)  // the fields stay on chip: Dtt u^n written once and read once per trial
+            h->stats.bytes_forward += kind == FWD_BORN ? cells * steps * Wv * (4.0 + 4.0 * nbw) : 0.0;
+        else if (tb2 && kind == FWD_BORN)
             h->stats.bytes_forward += cells * steps * Wv * (10.0 + 10.0 * nbw + (hist ? 4.0 : 0.0));
         else
             h->stats.bytes_forward += cells * steps * Wv *
@@ -2008,7 +2256,7 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
         if (need_ckpt) {
             if (!hist) {
                 h->stats.cell_updates_recompute += cells * steps * Wv;
-                h->stats.bytes_recompute += cells * steps * Wv * (tb2 ? 14.0 : 20.0);
+                h->stats.bytes_recompute += cells * steps * Wv * (rs.use ? 4.0 : tb2 ? 14.0 : 20.0);
             }
             h->stats.cell_updates_adjoint += cells * steps * Wv * nbw;
             // adjoint: per (shot, trial) mu^{n+1}, mu^{n+2}, write mu^n = 12 B; per shot Dtt 4 B;
@@ -2017,8 +2265,9 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
             //  Kahan fold of 20 B per cell once per segment)
             const bool seg3 = w.seg != nullptr;
             const double img_b = seg3 ? 8.0 + 20.0 / h->K : (h->kahan ? 16.0 : 8.0);
-            h->stats.bytes_adjoint += cells * steps * (12.0 * Wv * nbw + 4.0 * Wv +
-                                                       (double)jb.groups * (4.0 + img_b * nbw));
+            h->stats.bytes_adjoint += rs.use ? cells * steps * 4.0 * Wv * nbw
+                                             : cells * steps * (12.0 * Wv * nbw + 4.0 * Wv +
+                                                                (double)jb.groups * (4.0 + img_b * nbw));
         }
     }
     h->ev_base = 0;
@@ -2140,7 +2389,8 @@ extern "C" probe_status probe_forward_nonlinear(probe_t h, const float* m, float
         TRY(ensure_buf(h, h->stage_out, nd * 4));
         dd = (float*)h->stage_out.p;
     }
-    TRY(ensure_ws(h, plan_wave(h, 1, 0, 0), 1, 0, 0));
+    const int fits = res_fits(h, 0, 0);
+    TRY(ensure_ws(h, plan_wave(h, 1, 0, 0, fits), 1, 0, 0, fits));
     // positivity of m is the caller's responsibility; non-finite values are caught by the output check
     cudaError_t e = launch_make_s(md, h->d_m0, h->ws.s_tmp, h->nz, h->ny, h->nx, h->pad, h->P, h->F, h->Nz, h->Ny,
                                   h->Nx, (float)(h->dt * h->dt), st);
@@ -2181,7 +2431,8 @@ extern "C" probe_status probe_gradient(probe_t h, const float* m, const float* r
     }
     probe_status st_ = PROBE_OK;
     do {
-        st_ = ensure_ws(h, plan_wave(h, 1, 1, 0), 1, 1, 0);
+        const int fits = res_fits(h, 1, 0);
+        st_ = ensure_ws(h, plan_wave(h, 1, 1, 0, fits), 1, 1, 0, fits);
         if (st_ != PROBE_OK) break;
         cudaError_t e = launch_make_s(md, h->d_m0, h->ws.s_tmp, h->nz, h->ny, h->nx, h->pad, h->P, h->F, h->Nz,
                                       h->Ny, h->Nx, (float)(h->dt * h->dt), st);
@@ -2232,6 +2483,14 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
     bool any_host = false;
     reset_stats(h0);
     h0->tp.pending = 0;  // this call's times are formed below
+    int res = 1;  // every model on the resident kernels, or none
+    for (int k = 0; k < nmodels; ++k) res = res && res_fits(models[k], 1, 1);
+    std::vector<ResSet> rss(nmodels);
+    if (res)
+        for (int k = 0; k < nmodels; ++k) {
+            rss[k] = res_set(models[k], FWD_BORN, true, models[k]->ns, nb[k]);
+            res = res && rss[k].use;
+        }
     for (int k = 0; k < nmodels; ++k) {
         probe_t h = models[k];
         bool hin = false;
@@ -2244,7 +2503,7 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
             outs[k] = (float*)h->stage_out.p;
         }
         any_host = any_host || hin || host_out[k];
-        TRY(ensure_ws(h, h->ns, nb[k], 1, 1));  // every shot of every model resident
+        TRY(ensure_ws(h, h->ns, nb[k], 1, 1, res));  // every shot of every model resident
         Workspace& w = h->ws;
         CK(h, cudaMemsetAsync(w.dm, 0, (size_t)nb[k] * h->F * 4, st));
         cudaError_t e = launch_embed(dmd, w.dm, nb[k], h->nz, h->nx, 1, h->pad, h->Nz, h->Nx, 1, h->P, h->F, 1.0f, st);
@@ -2273,19 +2532,21 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
         key.push_back(jb.nb);
     }
     int grp = 0;
-    TRY(autotune_2d(h0, key, sw.jobs, FWD_BORN, true, true, st, &grp));
+    if (!res) TRY(autotune_2d(h0, key, sw.jobs, FWD_BORN, true, true, st, &grp));
     for (Job& jb : sw.jobs) {
         if (grp > 0) jb.shot_group = std::min(grp, jb.W);
+        if (res) jb.shot_group = 1;
         jb.groups = (jb.W + jb.shot_group - 1) / jb.shot_group;
         Workspace& w = jb.h->ws;
         CK(jb.h, cudaMemsetAsync(w.img, 0, (size_t)jb.groups * jb.nb * jb.h->F * 4, st));
         CK(jb.h, cudaMemsetAsync(w.comp, 0, (size_t)jb.groups * jb.nb * jb.h->F * 4, st));
     }
     h0->stats.shot_group = sw.jobs[0].shot_group;
-    h0->stats.pipeline_forward = h0->tile_z == kPipeTZ ? h0->opt_pipeline : 0;
-    h0->stats.pipeline_adjoint = h0->tile_z == kPipeTZ ? h0->pipe_adj : 0;
-    h0->stats.pipeline_rows = h0->tile_z == kPipeTZ ? h0->ws_rows : 0;
-    h0->stats.pipeline_rows_adjoint = h0->tile_z == kPipeTZ ? h0->ws_rows_adj : 0;
+    const bool piped = h0->tile_z == kPipeTZ && !res;
+    h0->stats.pipeline_forward = res ? 1 : (piped ? h0->opt_pipeline : 0);
+    h0->stats.pipeline_adjoint = res ? 1 : (piped ? h0->pipe_adj : 0);
+    h0->stats.pipeline_rows = piped ? h0->ws_rows : 0;
+    h0->stats.pipeline_rows_adjoint = piped ? h0->ws_rows_adj : 0;
     if (h0->opt_timing) TRY(ensure_events(h0, 3 + 2 * h0->nck + 2));
     // the whole group's sweeps as one graph (cached on h0 by handles, workspaces and variants)
     std::vector<long long> gkey = key;
@@ -2299,15 +2560,24 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
     gkey.push_back(h0->ws_rows_adj);
     gkey.push_back(h0->opt_timing);
     gkey.push_back(h0->tile_z);
+    gkey.push_back(res);
     long long cnt[4] = {0, 0, 0, 0};
     TRY(run_maybe_graph(h0, gkey, st, cnt, [&](cudaStream_t ss) -> probe_status {
         Sweep sw2;
         sw2.jobs = sw.jobs;
-        TRY(prepare_sweep(sw2, h0, ss));
-        record(h0, 0, ss);
-        TRY(run_forward(sw2, FWD_BORN, true));
-        record(h0, 1, ss);
-        TRY(run_adjoint(sw2));
+        if (res) {  // model after model
+            sw2.st = ss;
+            record(h0, 0, ss);
+            for (int k = 0; k < nmodels; ++k) TRY(run_forward_res(sw2, sw2.jobs[k], rss[k], FWD_BORN, true));
+            record(h0, 1, ss);
+            for (int k = 0; k < nmodels; ++k) TRY(run_adjoint_res(sw2, sw2.jobs[k], rss[k]));
+        } else {
+            TRY(prepare_sweep(sw2, h0, ss));
+            record(h0, 0, ss);
+            TRY(run_forward(sw2, FWD_BORN, true));
+            record(h0, 1, ss);
+            TRY(run_adjoint(sw2));
+        }
         cnt[0] = sw2.launches_fwd;
         cnt[1] = sw2.launches_rec;
         cnt[2] = sw2.launches_adj;
