@@ -309,6 +309,11 @@ def kernel_label(pipeline, adjoint, ndim=2, cluster=False, group=1, time_block=0
                      "summed in distributed shared memory before one Kahan update)" if adjoint else
                      "k_fwd3d_cl (incident + Born fields of a column tile on a cluster of 1 + p CTAs, "
                      "Dtt u0 exchanged in distributed shared memory)"), "stencil3d.cu")
+        if pipeline == 4:
+            return (("k_step3d_q<ADJ> (adjoint; the imaging terms of three steps added to the checkpoint-segment "
+                     "images every third step, Kahan fold per segment)" if adjoint else
+                     "k_step3d_q<BORN> / <INC> (3D forward steps, one field kind per launch, z taps in registers)"),
+                    "stencil3d_q.cu")
         ws = ("k_step3d_ws" if pipeline == 2 else "k_step3d_ws[last-warp refill]" if pipeline == 3
               else "k_step3d")
         return ((f"{ws}<ADJ> (adjoint + imaging into checkpoint-segment images, Kahan fold per segment)"

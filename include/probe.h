@@ -122,8 +122,8 @@ typedef enum {
                                     kernels; 2 = pipelined kernels whose ring is refilled by a
                                     producer warp; 3 = pipelined kernels whose ring slot is refilled
                                     by the last compute warp done with it (no producer warp); by
-                                    default the 3D autotuner picks 2 or 3, for the forward and the
-                                    adjoint.  Setting it turns that choice off. */
+                                    default the 3D kernels keep the z taps in registers (reported as
+                                    4).  Every 3D family gives the same bits. */
     PROBE_OPT_DTT_HISTORY = 8,   /* 2D: 1 = keep Dtt u^n of every step in device memory instead of
                                     checkpointing and recomputing (FP32, W (nt-1) planes); 0 (default) */
     PROBE_OPT_AUTOTUNE = 9,      /* 1 (default): 2D grids that fit a cluster's shared memory run on the
@@ -190,7 +190,7 @@ typedef struct {
     int pipeline_forward;        /* 2D forward kernel: 0 one tile per CTA, 1 cluster-resident (one
                                     launch per field kind and checkpoint segment), 2..4 pipeline stages;
                                     3D: 0 one barrier per plane, 2 producer-warp refill, 3 refill by
-                                    the last compute warp */
+                                    the last compute warp, 4 z taps in a register queue */
     int pipeline_adjoint;        /* 2D adjoint kernel: same encoding; 3D: as the forward, for the
                                     adjoint with the receiver injection from a per-segment band
                                     buffer */

@@ -55,10 +55,10 @@ struct TunedEntry {
     int pipe_fwd = 2, pipe_adj = 2, group = 4, rows = 2, rows_adj = 1, tblock = 1;
 };
 
-// 3D autotuner result: refill scheme of the pipelined forward and adjoint kernels, planes per CTA.
+// 3D autotuner result: planes per CTA.
 struct Tuned3 {
     std::vector<long long> key;  // kind, adjoint, shots, trials
-    int fam_fwd = 2, fam_inc = 2, fam_adj = 2, zc = 64;
+    int zc = 64;
 };
 
 // Cluster-resident 2D kernels for one workload (shots, trials, adjoint): cluster sizes of each field

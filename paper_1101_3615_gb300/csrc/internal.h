@@ -115,6 +115,11 @@ enum Step3Mode { STEP3_INC = 0, STEP3_INC_SAMPLE = 1, STEP3_BORN = 2, STEP3_ADJ 
 
 struct alignas(128) ModelStep3D {
     CUtensorMap tm;    // 4D map (x, y, z, volume) over the state being differentiated
+    // register-queue kernels, plain 64 x 16 boxes: the state (older level), s, the Dtt buffer (volume
+    // shot * d_slots + d_slot), dm (Born) or the image [shot][trial] (adjoint)
+    CUtensorMap tm_prev, tm_s, tm_d, tm_own;
+    int d_slots, d_slot;
+    int shots_inner;     // CTA order: the shots of a column tile run together (1) or one shot after the other (0)
     int Nz, Ny, Nx, P, pad, nz, ny, nx;
     int tiles_x, tiles_y, zchunks, ZC;
     int nshots, nfield;  // fields per shot in this launch (1 incident, nb Born / adjoint)
@@ -153,6 +158,7 @@ struct alignas(128) ModelStep3D {
 
 struct StepParams3D {
     int n, nt;
+    float one;  // 1, unknown to the compiler (register-queue kernels; set by their launcher)
     int* err;
     ModelStep3D m;
     ModelStep3D m2;  // cluster kernels: the Born fields of the fused forward step
@@ -160,6 +166,8 @@ struct StepParams3D {
 
 // pipeline: 0 one barrier per plane; 2 producer warp; 3 the last compute warp out of a slot refills it
 cudaError_t launch_step3d(int mode, bool kahan, int pipeline, const StepParams3D& p, cudaStream_t st);
+// Register-queue kernels (stencil3d_q.cu); terms: imaging terms added by an adjoint step (0 to 3).
+cudaError_t launch_step3d_q(int mode, int terms, const StepParams3D& p, cudaStream_t st);
 size_t step3d_smem_bytes();
 // Fused incident + Born step on clusters of 1 + nb CTAs (m: incident, m2: Born, nb = m2.nfield <= 7).
 cudaError_t launch_fwd3d_cluster(const StepParams3D& p, cudaStream_t st);

@@ -150,6 +150,21 @@ probe_status encode_plain(probe_t h, CUtensorMap* map, const float* base, int pl
     return PROBE_OK;
 }
 
+// 3D FP32 tensor map over `vols` volumes with a plain 64 x 16 one-plane box (no halo).
+probe_status encode_plain3(probe_t h, CUtensorMap* map, const float* base, int vols) {
+    TRY(get_encoder(h));
+    cuuint32_t es[4] = {1, 1, 1, 1};
+    cuuint64_t dims[4] = {(cuuint64_t)h->Nx, (cuuint64_t)h->Ny, (cuuint64_t)h->Nz, (cuuint64_t)vols};
+    cuuint64_t strides[3] = {(cuuint64_t)h->P * 4, (cuuint64_t)h->Ny * h->P * 4, (cuuint64_t)h->F * 4};
+    cuuint32_t box[4] = {(cuuint32_t)kTX, (cuuint32_t)kTY3D, 1, 1};
+    CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(base), dims, strides, box, es,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS)
+        return fail(h, PROBE_ERR_CUDA, "cuTensorMapEncodeTiled (3D plain box) failed (" + std::to_string((int)r) + ")");
+    return PROBE_OK;
+}
+
 // Workspace generations are unique in the process, so a cached graph keyed by
 // (handle, generation) can never match a later workspace at reused addresses.
 std::atomic<long long> g_generation{0};
@@ -1133,6 +1148,27 @@ void fill3d(const Job& jb, ModelStep3D& m) {
     m.comp = w.comp;
 }
 
+// Operand maps of the register-queue kernels: the state's plain boxes, s, the Dtt buffer, and dm (Born)
+// or the image that the adjoint adds to (own, vols volumes; null: none).
+probe_status fill3d_q(const Job& jb, ModelStep3D& m, const float* own, int vols, int shots_inner) {
+    probe_t h = jb.h;
+    Workspace& w = h->ws;
+    TRY(encode_plain3(h, &m.tm_prev, m.state, jb.W * m.nvol_shot));
+    TRY(encode_plain3(h, &m.tm_s, jb.s, 1));
+    if (w.dtt) TRY(encode_plain3(h, &m.tm_d, w.dtt, w.W * w.dtt_slots));
+    if (own) TRY(encode_plain3(h, &m.tm_own, own, vols));
+    m.d_slots = w.dtt_slots;
+    m.shots_inner = shots_inner;
+    return PROBE_OK;
+}
+
+// One 3D step launch: pipeline 4 = register-queue kernels (terms: imaging terms of an adjoint step), else
+// as launch_step3d.
+cudaError_t step3(int mode, bool kahan, int pipeline, const StepParams3D& p, cudaStream_t st, int terms = 1) {
+    if (pipeline == 4 && !(mode == STEP3_ADJ && kahan)) return launch_step3d_q(mode, terms, p, st);
+    return launch_step3d(mode, kahan, pipeline, p, st);
+}
+
 struct Count3 {
     long long fwd = 0, rec = 0, adj = 0, other = 0;
 };
@@ -1141,39 +1177,33 @@ probe_status launch3(probe_t h, int mode, StepParams3D& p, int n, cudaStream_t s
     p.n = n;
     // the incident step (forward and recompute) may use its own ring-refill scheme
     const int pipe = (mode == STEP3_INC || mode == STEP3_INC_SAMPLE) ? h->pipe_inc : h->opt_pipeline;
-    cudaError_t e = launch_step3d(mode, h->kahan != 0, pipe, p, st);
+    cudaError_t e = step3(mode, h->kahan != 0, pipe, p, st);
     if (e != cudaSuccess) return cuda_fail(h, e, what);
     return PROBE_OK;
 }
 
 // 3D autotuner, on the first call for a workload key, timed on the real workspace (round-robin
 // over three rounds, each candidate's fastest round kept): the z planes one CTA marches (32, 64,
-// 128) with the ring-refill scheme of the pipelined forward kernels (2: producer warp, 3: the
-// last compute warp out of a slot) on one incident and (for the Born forward) one Born launch per
-// candidate; then, for calls with an adjoint sweep, the refill scheme of the adjoint on one
-// adjoint launch per scheme.  The launches write only the state planes, the Dtt plane and the
-// segment image or the image, which the call clears or rewrites before it reads them.  None of
-// the choices changes a result.
+// 128) on one incident and (for the Born forward) one Born launch per candidate.  The launches write
+// only the state planes and the Dtt plane, which the call clears or rewrites before it reads them.
+// The choice does not change a result.  The kernels are the register-queue ones (pipeline 4) unless the
+// caller chose another family: those were faster in every launch of every grid timed (per step, us:
+// 4 x 168^3 incident 94 against 107 and two Born fields 152 against 187; 8 x 296^3 743 against 786 and four
+// Born fields 2660 against 3120, their adjoint 3290 against 3890 with the fold of the segment images).
 probe_status autotune_3d(const Job& jb, FwdKind kind, bool adjoint, cudaStream_t st) {
     probe_t h = jb.h;
-    const bool fam_fixed = h->user_fixed || h->opt_pipeline == 0;
-    if (h->ndim != 3 || (h->user_zc3d && fam_fixed) || h->opt_cluster3d) return PROBE_OK;
+    if (h->ndim != 3 || h->user_zc3d || h->opt_cluster3d) return PROBE_OK;
     const std::vector<long long> key = {(long long)kind, (long long)adjoint, jb.W, jb.nb};
     for (const Tuned3& t : h->tuned3)
         if (t.key == key) {
-            if (!h->user_zc3d) h->zc3d = t.zc;
-            if (!fam_fixed) {
-                h->opt_pipeline = t.fam_fwd;
-                h->pipe_inc = t.fam_inc;
-                h->pipe_adj = t.fam_adj;
-            }
+            h->zc3d = t.zc;
             return PROBE_OK;
         }
     if (!h->opt_autotune) return PROBE_OK;
     Workspace& w = h->ws;
     if (!w.dtt) return PROBE_OK;
     const bool born = kind == FWD_BORN;
-    StepParams3D pi, pb, pa;
+    StepParams3D pi, pb;
     fill3d(jb, pi.m);
     pi.nt = h->nt;
     pi.err = h->d_err;
@@ -1183,7 +1213,7 @@ probe_status autotune_3d(const Job& jb, FwdKind kind, bool adjoint, cudaStream_t
     pi.m.nvol_shot = 2;
     pi.m.Dout = w.dtt;
     pi.m.Dout_shot_stride = dtt_stride3(h);
-    fill3d(jb, pb.m);  // Born fields (forward) and adjoint fields share the f planes
+    fill3d(jb, pb.m);
     pb.nt = h->nt;
     pb.err = h->d_err;
     pb.m.tm = w.tm_f;
@@ -1192,11 +1222,8 @@ probe_status autotune_3d(const Job& jb, FwdKind kind, bool adjoint, cudaStream_t
     pb.m.nvol_shot = 2 * jb.nb;
     pb.m.Din = w.dtt;
     pb.m.Din_shot_stride = dtt_stride3(h);
-    pa = pb;  // adjoint: no receiver injection (rrow null); a segment's first step writes its image
-    if (w.seg) {
-        pa.m.img = w.seg;
-        pa.m.seg_first = 1;
-    }
+    TRY(fill3d_q(jb, pi.m, nullptr, 0, 1));
+    TRY(fill3d_q(jb, pb.m, w.dm, std::max(jb.nb, 1), 1));
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t ce = cudaEventCreate(&e0);
     if (ce == cudaSuccess) ce = cudaEventCreate(&e1);
@@ -1217,87 +1244,37 @@ probe_status autotune_3d(const Job& jb, FwdKind kind, bool adjoint, cudaStream_t
         *best = std::min(*best, ms);
         return PROBE_OK;
     };
-    auto set_zc = [&](int zc) {
-        for (StepParams3D* q : {&pi, &pb, &pa}) {
-            q->m.ZC = zc;
-            q->m.zchunks = (h->Nz + zc - 1) / zc;
-        }
-    };
-    // forward: (refill scheme, planes), the incident and the Born launches timed apart so that
-    // each gets its own scheme; the caller's fixed choices stay fixed
-    std::vector<int> fams = {2, 3}, zcs = {32, 64, 128};
-    if (fam_fixed) fams = {h->opt_pipeline};
-    if (h->user_zc3d) zcs = {h->zc3d};
-    std::vector<std::pair<int, int>> cand;
-    for (int fam : fams)
-        for (int zc : zcs) cand.push_back({fam, zc});
-    const int nc = (int)cand.size();
-    std::vector<float> t_inc(nc, 1e30f), t_born(nc, born ? 1e30f : 0.f);
+    const std::vector<int> zcs = {32, 64, 128};
+    std::vector<float> t_inc(zcs.size(), 1e30f), t_born(zcs.size(), born ? 1e30f : 0.f);
     probe_status ps = PROBE_OK;
     for (int round = 0; round < 3 && ps == PROBE_OK; ++round)
-        for (int c = 0; c < nc && ps == PROBE_OK; ++c) {
-            set_zc(cand[c].second);
+        for (size_t c = 0; c < zcs.size() && ps == PROBE_OK; ++c) {
+            for (StepParams3D* q : {&pi, &pb}) {
+                q->m.ZC = zcs[c];
+                q->m.zchunks = (h->Nz + zcs[c] - 1) / zcs[c];
+            }
             for (int mode : {STEP3_INC, STEP3_BORN}) {
                 if (ps != PROBE_OK || (mode == STEP3_BORN && !born)) continue;
                 StepParams3D& q = (mode == STEP3_INC) ? pi : pb;
                 ps = timed(mode == STEP3_INC ? &t_inc[c] : &t_born[c], [&]() -> probe_status {
-                    for (int n = 0; n < 2; ++n) {
-                        q.n = n;
-                        cudaError_t e = launch_step3d(mode, false, cand[c].first, q, st);
-                        if (e != cudaSuccess) return cuda_fail(h, e, "autotuner launch");
-                    }
+                    for (int n = 0; n < 2; ++n) TRY(launch3(h, mode, q, n, st, "autotuner launch"));
                     return PROBE_OK;
                 });
             }
         }
-    // per plane count the faster scheme of each launch; then the plane count of the fastest step
-    int zc = h->zc3d, fam_inc = fams[0], fam_fwd = fams[0];
+    int zc = h->zc3d;
     float best_step = 1e30f;
-    for (int z : zcs) {
-        int bi = -1, bb = -1;
-        for (int c = 0; c < nc; ++c) {
-            if (cand[c].second != z) continue;
-            if (bi < 0 || t_inc[c] < t_inc[bi]) bi = c;
-            if (bb < 0 || t_born[c] < t_born[bb]) bb = c;
+    for (size_t c = 0; c < zcs.size(); ++c)
+        if (t_inc[c] + t_born[c] < best_step) {
+            best_step = t_inc[c] + t_born[c];
+            zc = zcs[c];
         }
-        if (bi >= 0 && t_inc[bi] + t_born[bb] < best_step) {
-            best_step = t_inc[bi] + t_born[bb];
-            zc = z;
-            fam_inc = cand[bi].first;
-            fam_fwd = cand[bb].first;
-        }
-    }
-    // adjoint refill scheme at the chosen planes
-    int fam_adj = fam_fixed ? h->pipe_adj : fam_fwd;
-    if (ps == PROBE_OK && adjoint && !fam_fixed && adj3d_ws(h)) {
-        float ba[2] = {1e30f, 1e30f};
-        set_zc(zc);
-        for (int round = 0; round < 3 && ps == PROBE_OK; ++round)
-            for (int c = 0; c < 2 && ps == PROBE_OK; ++c)
-                ps = timed(&ba[c], [&]() -> probe_status {
-                    for (int n = 0; n < 2; ++n) {
-                        pa.n = h->nt - 1 - n;
-                        cudaError_t e = launch_step3d(STEP3_ADJ, false, 2 + c, pa, st);
-                        if (e != cudaSuccess) return cuda_fail(h, e, "autotuner launch");
-                    }
-                    return PROBE_OK;
-                });
-        fam_adj = (ba[1] < ba[0]) ? 3 : 2;
-    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     TRY(ps);
     h->zc3d = zc;
-    if (!fam_fixed) {
-        h->opt_pipeline = born ? fam_fwd : fam_inc;
-        h->pipe_inc = fam_inc;
-        h->pipe_adj = fam_adj;
-    }
     Tuned3 t;
     t.key = key;
-    t.fam_fwd = h->opt_pipeline;
-    t.fam_inc = h->pipe_inc;
-    t.fam_adj = h->pipe_adj;
     t.zc = h->zc3d;
     h->tuned3.push_back(t);
     return PROBE_OK;
@@ -1329,7 +1306,9 @@ probe_status run_forward3d(const Job& jb, FwdKind kind, bool ckpt, cudaStream_t 
         pb.m.nvol_shot = 2 * jb.nb;
         pb.m.Din = w.dtt;
         pb.m.Din_shot_stride = dtt_stride3(h);
+        TRY(fill3d_q(jb, pb.m, w.dm, jb.nb, 1));
     }
+    TRY(fill3d_q(jb, pi.m, nullptr, 0, 1));
     const int imode = (kind == FWD_INCIDENT_SAMPLE) ? STEP3_INC_SAMPLE : STEP3_INC;
     // fused incident + Born step on thread-block clusters (Dtt u0 exchanged in shared memory)
     const bool fused = born && (h->opt_cluster3d & 1) && jb.nb + 1 <= 8;
@@ -1381,6 +1360,7 @@ probe_status run_forward3d(const Job& jb, FwdKind kind, bool ckpt, cudaStream_t 
                 CK(h, cudaStreamWaitEvent(sb, h->ov_inc[slot], 0));
             }
             pb.m.Din = w.dtt + (long long)slot * h->F;
+            pb.m.d_slot = slot;
             TRY(launch3(h, STEP3_BORN, pb, n, sb, "Born step launch"));
             if (overlap) CK(h, cudaEventRecord(h->ov_born[slot], sb));
             c.fwd++;
@@ -1434,6 +1414,8 @@ probe_status run_adjoint3d(const Job& jb, cudaStream_t st, Count3& c) {
         pa.m.inj = (h->nband > 0) ? w.inj : nullptr;
         pa.m.inj_block = block;
     }
+    TRY(fill3d_q(jb, pi.m, nullptr, 0, 1));
+    TRY(fill3d_q(jb, pa.m, w.seg ? w.seg : w.img, jb.W * jb.nb, 0));
     int ev = 2;
     for (int k = h->nck - 1; k >= 0; --k) {
         const int k0 = k * h->K;
@@ -1461,6 +1443,7 @@ probe_status run_adjoint3d(const Job& jb, cudaStream_t st, Count3& c) {
         }
         for (int n = k1; n >= k0 + 1; --n) {
             pa.m.Din = w.dtt + (long long)(n - 1 - k0) * h->F;
+            pa.m.d_slot = n - 1 - k0;
             if (clustered) {
                 pa.n = n;
                 pa.m.inj_slot = k1 - n;
@@ -1471,11 +1454,18 @@ probe_status run_adjoint3d(const Job& jb, cudaStream_t st, Count3& c) {
                 // Kahan across segments; without: plain FP32 into the image itself
                 pa.n = n;
                 pa.m.inj_slot = k1 - n;
+                // register-queue kernels: the image every third step, with the terms of the three
+                const int pipe = ws ? h->pipe_adj : 0;
+                int terms = 1;
+                if (pipe == 4) {
+                    const int j = (k1 - n) % 3;
+                    terms = (j == 2 || n == k0 + 1) ? j + 1 : 0;
+                }
                 if (w.seg) {
                     pa.m.img = w.seg;
-                    pa.m.seg_first = (n == k1) ? 1 : 0;
+                    pa.m.seg_first = (n + terms - 1 == k1) ? 1 : 0;
                 }
-                cudaError_t e = launch_step3d(STEP3_ADJ, !w.seg && h->kahan != 0, ws ? h->pipe_adj : 0, pa, st);
+                cudaError_t e = step3(STEP3_ADJ, !w.seg && h->kahan != 0, pipe, pa, st, terms);
                 if (e != cudaSuccess) return cuda_fail(h, e, "adjoint step launch");
             }
             c.adj++;
@@ -1645,6 +1635,7 @@ extern "C" probe_status probe_create(probe_t* out, const probe_grid* g, const fl
     h->kahan = g->kahan ? 1 : 0;
     h->K = g->ckpt_stride > 0 ? g->ckpt_stride : (int)std::ceil(std::sqrt((double)nt));
     h->K = std::max(1, std::min(h->K, nt - 1));
+    if (D == 3) h->opt_pipeline = h->pipe_inc = h->pipe_adj = 4;
     h->nck = (nt - 2) / h->K + 1;  // checkpoints at n = 0, K, ... < nt - 1
 
     auto bad = [&](const std::string& m) {
@@ -2177,7 +2168,7 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
             h->stats.pipeline_adjoint = rs.use ? 1 : (piped ? h->pipe_adj : 0);
             if (h->ndim == 3) TRY(autotune_3d(jb, kind, need_ckpt, st));
             h->stats.planes_3d = (h->ndim == 3) ? h->zc3d : 0;
-            if (h->ndim == 3) {  // 0 one barrier per plane, 2 producer warp, 3 refill by the last compute warp
+            if (h->ndim == 3) {  // 0 one barrier per plane, 2 producer warp, 3 last compute warp, 4 register queue
                 h->stats.pipeline_forward = !(h->opt_cluster3d & 1) ? h->opt_pipeline : 0;
                 h->stats.pipeline_incident = !(h->opt_cluster3d & 1) ? h->pipe_inc : 0;
                 h->stats.pipeline_adjoint = (adj3d_ws(h) && (h->nband == 0 || w.inj)) ? h->pipe_adj : 0;
