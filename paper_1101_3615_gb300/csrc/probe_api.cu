@@ -283,7 +283,7 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, i
     const int G = W;  // image groups for the smallest shot group: any group size fits
     const int history = use_history(h, with_ckpt) ? 1 : 0;
     const int slots2 = h->ndim == 2 ? dtt_slots_2d(h, with_ckpt, history, res) : 0;
-    if (w.u && (h->ndim == 3 || w.dtt_slots == slots2) && w.W >= W && w.nb >= nb && w.with_ckpt >= with_ckpt && w.with_data >= with_data &&
+    if (w.u && (h->ndim == 3 || w.dtt_slots >= slots2) && w.W >= W && w.nb >= nb && w.with_ckpt >= with_ckpt && w.with_data >= with_data &&
         w.groups >= G && w.tm_tile_z == h->tile_z && w.W == W && w.nb == nb && w.history == history)
         return PROBE_OK;
     free_ws(w);
