@@ -23,7 +23,8 @@
 // There is no CTA-wide barrier in the main loop; a sentinel descriptor ends
 // the list.  Every wait is bounded (2 s of %globaltimer) and reports through
 // the device error word.  The arithmetic is that of stencil2d.cu operation for
-// operation, so both kernel families give the same bits.
+// operation; on all-interior tiles the compiler fuses the packed multiply and add of the
+// leapfrog, so there the two families differ by rounding (about 2e-7), elsewhere not at all.
 #include "common.cuh"
 #include "internal.h"
 
@@ -88,9 +89,10 @@ __device__ __forceinline__ float cell_update(const ModelStep2D& M, bool fast, in
 //   sum_k w_k (v_{c+k} + v_{c-k} - 2 v_c) = sum_{m=0..3} C_m (d_{c+m} - d_{c-m-1}),
 //   C_m = sum_{k>m} w_k / h^2,
 // x first (11 shared differences per row), then z (R + 7 shared differences per column).
-// PACKED: z taps in packed FP32x2 (the forward kernels) or scalar (the adjoint, where the packed
-// form measured slower); the two give the same bits.
-template <int R, bool PACKED>
+// The z taps in packed FP32x2: the scalar form's subtractions and fused multiply-adds, two lanes an
+// instruction, the same bits.  The adjoint kernel took the scalar form while it was held to 2 CTAs
+// per SM (packed: no difference there); see k_adj2d_ws for the two together.
+template <int R>
 __device__ __forceinline__ void lap_rows(const float* t, int row, int col, const ModelStep2D& M, float4 c[R],
                                          float L[R][4]) {
     const float* rp = t + row * HX + col;
@@ -113,45 +115,6 @@ __device__ __forceinline__ void lap_rows(const float* t, int row, int col, const
     // z, outward: rows below the first cell row (lo) and above the last (hi) are loaded
     // as the tap index m grows; row r's term m is C_m ((v_{r+m+1} - v_{r+m}) - (v_{r-m} - v_{r-m-1})).
     // Differences between rows inside the block are formed once and shared by the R rows.
-    if (!PACKED) {
-        if (R == 1) {
-            float4 lo = c[0], hi = c[0];
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const float4 dn = ld4(rp - (m + 1) * HX), up = ld4(rp + (m + 1) * HX);
-                L[0][0] = fmaf(M.czm[m], (up.x - hi.x) - (lo.x - dn.x), L[0][0]);
-                L[0][1] = fmaf(M.czm[m], (up.y - hi.y) - (lo.y - dn.y), L[0][1]);
-                L[0][2] = fmaf(M.czm[m], (up.z - hi.z) - (lo.z - dn.z), L[0][2]);
-                L[0][3] = fmaf(M.czm[m], (up.w - hi.w) - (lo.w - dn.w), L[0][3]);
-                lo = dn;
-                hi = up;
-            }
-        } else {
-            const float4 c0 = c[0], c1 = c[R - 1];
-            const float4 gin = make_float4(c1.x - c0.x, c1.y - c0.y, c1.z - c0.z, c1.w - c0.w);
-            float4 lo = c0, hi = c1, glo = gin, ghi = gin;
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const float4 dn = ld4(rp - (m + 1) * HX), up = ld4(rp + (m + 2) * HX);
-                const float4 gd = make_float4(lo.x - dn.x, lo.y - dn.y, lo.z - dn.z, lo.w - dn.w);
-                const float4 gu = make_float4(up.x - hi.x, up.y - hi.y, up.z - hi.z, up.w - hi.w);
-                L[0][0] = fmaf(M.czm[m], ghi.x - gd.x, L[0][0]);
-                L[0][1] = fmaf(M.czm[m], ghi.y - gd.y, L[0][1]);
-                L[0][2] = fmaf(M.czm[m], ghi.z - gd.z, L[0][2]);
-                L[0][3] = fmaf(M.czm[m], ghi.w - gd.w, L[0][3]);
-                L[R - 1][0] = fmaf(M.czm[m], gu.x - glo.x, L[R - 1][0]);
-                L[R - 1][1] = fmaf(M.czm[m], gu.y - glo.y, L[R - 1][1]);
-                L[R - 1][2] = fmaf(M.czm[m], gu.z - glo.z, L[R - 1][2]);
-                L[R - 1][3] = fmaf(M.czm[m], gu.w - glo.w, L[R - 1][3]);
-                lo = dn;
-                hi = up;
-                glo = gd;
-                ghi = gu;
-            }
-        }
-        return;
-    }
-    // (packed: the same subtractions and fused multiply-adds, two lanes per instruction)
     if (R == 1) {
         P4 acc = p4(L[0][0], L[0][1], L[0][2], L[0][3]);
         P4 lo = p4(c[0]), hi = lo;
@@ -335,7 +298,7 @@ __global__ void __launch_bounds__(kWsThreads, R == 1 ? 4 : 3) k_fwd2d_ws(const _
         const bool fast = q.fast != 0;
         float L[R][4];
         float4 c[R];
-        lap_rows<R, true>(st, lz + 4, lx + 4, M, c, L);
+        lap_rows<R>(st, lz + 4, lx + 4, M, c, L);
         if (q.f == 0) {
 #pragma unroll
             for (int r = 0; r < R; ++r) {
@@ -410,8 +373,15 @@ __global__ void __launch_bounds__(kWsThreads, R == 1 ? 4 : 3) k_fwd2d_ws(const _
 // ---- adjoint ---------------------------------------------------------------
 // Item = (model, shot group, tile); its groups are (shot jj of the group, trial bi of the chunk),
 // jj-major.  s is staged with the item's first group, Dtt with each shot's first trial.
+// Bound: issue slots and load latency together (not DRAM: the levels of 32 shots of 541^2
+// stay in L2).  So the kernel asks for registers that let 4 (one trial) or 3 (two and more) CTAs
+// of one row per thread sit on an SM, instead of 2, and takes the z taps in packed FP32x2.  us per
+// time step, before -> after: 32 shots of 541^2, one trial 43.3 -> 40.9; gradient, 8 shots of 1041^2
+// 37.3 -> 35.3; group of 341^2, 541^2 and 741^2, 8 shots x 4 trials each 158 -> 144.
+constexpr int adj_ctas(int nbc, int r) { return nbc * r >= 8 ? 1 : r == 2 ? 2 : nbc == 1 ? 4 : 3; }
+
 template <int NBC, bool KAHAN, int S, bool MULTI, int R>
-__global__ void __launch_bounds__(kWsThreads, (NBC * R >= 8) ? 1 : 2) k_adj2d_ws(const __grid_constant__ StepParams2D p) {
+__global__ void __launch_bounds__(kWsThreads, adj_ctas(NBC, R)) k_adj2d_ws(const __grid_constant__ StepParams2D p) {
     using T = Ws<R>;
     extern __shared__ __align__(128) float smem[];
     __shared__ __align__(8) uint64_t full[S], empty[S];
@@ -534,7 +504,7 @@ __global__ void __launch_bounds__(kWsThreads, (NBC * R >= 8) ? 1 : 2) k_adj2d_ws
         }
         float L[R][4];
         float4 c[R];
-        lap_rows<R, false>(st, lz + 4, lx + 4, M, c, L);
+        lap_rows<R>(st, lz + 4, lx + 4, M, c, L);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int z = q.z0 + lz + r;
