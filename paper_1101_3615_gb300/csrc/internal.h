@@ -208,7 +208,9 @@ struct ResParams2D {
     float cxm[4], czm[4];
     float inv_dt2, vol_inv;
     long long F;
-    float* state;        // [nshots][nfield][2][F]
+    const float* in;     // [nshots][nfield][2][F]: the two levels before the launch, the newer in plane pin
+    float* out;          // the same after it, the newest in plane pout; may be `in`, or null (not wanted)
+    int pin, pout;
     const float* s;
     const float* dm;     // Born: [nfield][F]
     float* dtt;          // Dtt u^n of level n: slot slot0 + k (forward), slot0 - k (adjoint, Dtt u^{n-1}); may be null (incident)

@@ -322,8 +322,10 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, i
     }
     TRY(alloc((void**)&w.s_tmp, (size_t)F * 4));
     TRY(alloc((void**)&w.src_wave, (size_t)W * 3 * 4));
-    if (with_ckpt && h->nband > 0 && (h->ndim == 2 || (h->opt_cluster3d & 2) || adj3d_ws(h)))  // one segment of adjoint injection
-        TRY(alloc((void**)&w.inj, (size_t)h->K * W * std::max(nb, 1) * inj_block(h) * 4));
+    // one segment of adjoint injection (two for the resident kernels)
+    if (with_ckpt && h->nband > 0 && (h->ndim == 2 || (h->opt_cluster3d & 2) || adj3d_ws(h)))
+        TRY(alloc((void**)&w.inj, (size_t)(slots2 > h->K && !history ? 2 : 1) * h->K * W * std::max(nb, 1) *
+                                      inj_block(h) * 4));
     // field planes must read as zero outside what the kernels write
     CK(h, cudaMemset(w.u, 0, (size_t)W * 2 * F * 4));
     CK(h, cudaMemset(w.f, 0, (size_t)W * std::max(nb, 1) * 2 * F * 4));
@@ -924,16 +926,20 @@ probe_status run_forward_res(Sweep& sw, Job& jb, const ResSet& rs, FwdKind kind,
     Workspace& w = h->ws;
     cudaStream_t st = sw.st;
     const bool born = kind == FWD_BORN;
-    CK(h, cudaMemsetAsync(w.u, 0, (size_t)jb.W * 2 * h->F * 4, st));
+    // FP32 checkpoints are the incident field's state itself: a segment reads its own checkpoint and
+    // writes the next one's.  16-bit ones are encoded from w.u.
+    const size_t per = ckpt ? (size_t)jb.W * ckpt_bytes_per_shot(h->snap, h->F) : 0;
+    const bool in_place = ckpt && h->snap == PROBE_SNAP_FP32;
+    CK(h, cudaMemsetAsync(in_place ? w.ckpt : (void*)w.u, 0, (size_t)jb.W * 2 * h->F * 4, st));
     if (born) CK(h, cudaMemsetAsync(w.f, 0, (size_t)jb.W * jb.nb * 2 * h->F * 4, st));
     ResParams2D pi, pb;
     fill_res(jb, pi);
     pi.nfield = 1;
-    pi.state = w.u;
+    pi.in = pi.out = w.u;
     if (kind == FWD_INCIDENT_SAMPLE) pi.data = jb.data;
     fill_res(jb, pb);
     pb.nfield = jb.nb;
-    pb.state = w.f;
+    pb.in = pb.out = w.f;
     pb.dm = w.dm;
     pb.dtt = w.dtt;
     pb.data = jb.data;
@@ -947,8 +953,13 @@ probe_status run_forward_res(Sweep& sw, Job& jb, const ResSet& rs, FwdKind kind,
     for (int n = 0, i = 0; n < h->nt - 1; n += h->K, ++i) {
         const int T = std::min(h->K, h->nt - 1 - n), set = i & 1;
         if (born && i >= 2) CK(h, cudaStreamWaitEvent(su, h->ov_born[set], 0));
-        if (ckpt) {
-            const size_t per = (size_t)jb.W * ckpt_bytes_per_shot(h->snap, h->F);
+        pi.pin = pb.pin = n & 1;
+        pi.pout = pb.pout = (n + T) & 1;
+        if (in_place) {
+            pi.in = (const float*)((const char*)w.ckpt + i * per);
+            pi.pin = pi.pout = 0;  // u^n first
+            pi.out = n + T < h->nt - 1 ? (float*)((char*)w.ckpt + (i + 1) * per) : nullptr;
+        } else if (ckpt) {
             cudaError_t e = launch_encode_ckpt(w.u, jb.W * 2, h->F, 2, n & 1, (n & 1) ^ 1, (char*)w.ckpt + i * per,
                                                w.scales + (size_t)i * jb.W * 2, h->snap, w.absmax, su);
             if (e != cudaSuccess) return cuda_fail(h, e, "checkpoint store");
@@ -987,17 +998,18 @@ probe_status run_adjoint_res(Sweep& sw, Job& jb, const ResSet& rs) {
     ResParams2D pi, pa;
     fill_res(jb, pi);
     pi.nfield = 1;
-    pi.state = w.u;
+    pi.in = w.u;
     pi.dtt = w.dtt;
     fill_res(jb, pa);
     pa.nfield = jb.nb;
-    pa.state = w.f;
+    pa.in = pa.out = w.f;
     pa.dtt = w.dtt;
     pa.rrow = h->nband > 0 ? h->d_rrow : nullptr;
-    pa.inj = w.inj;
     pa.inj_block = inj_block(h);
     pa.img = w.img;
     pa.comp = w.comp;
+    const size_t per = (size_t)jb.W * ckpt_bytes_per_shot(h->snap, h->F);
+    const long long inj_seg = (long long)h->K * jb.W * jb.nb * pa.inj_block;
     TRY(ensure_overlap_stream(h));
     cudaStream_t su = h->ostream;
     CK(h, cudaEventRecord(h->ov_inc[0], st));
@@ -1008,11 +1020,26 @@ probe_status run_adjoint_res(Sweep& sw, Job& jb, const ResSet& rs) {
         if (k0 >= k1) continue;
         record(h, ev++, st);
         if (i >= 2) CK(h, cudaStreamWaitEvent(su, h->ov_born[set], 0));
-        const size_t per = (size_t)jb.W * ckpt_bytes_per_shot(h->snap, h->F);
-        cudaError_t e = launch_decode_ckpt((const char*)w.ckpt + (size_t)k * per, w.scales + (size_t)k * jb.W * 2,
-                                           jb.W * 2, h->F, 2, k0 & 1, (k0 & 1) ^ 1, h->snap, w.u, su);
-        if (e != cudaSuccess) return cuda_fail(h, e, "checkpoint restore");
-        sw.launches_other += codec_launches(h->snap, false, 2, k0 & 1);
+        cudaError_t e = cudaSuccess;
+        if (h->snap == PROBE_SNAP_FP32) {
+            pi.in = (const float*)((const char*)w.ckpt + (size_t)k * per);
+            pi.pin = 0;
+        } else {
+            e = launch_decode_ckpt((const char*)w.ckpt + (size_t)k * per, w.scales + (size_t)k * jb.W * 2, jb.W * 2, h->F,
+                                   2, k0 & 1, (k0 & 1) ^ 1, h->snap, w.u, su);
+            if (e != cudaSuccess) return cuda_fail(h, e, "checkpoint restore");
+            sw.launches_other += codec_launches(h->snap, false, 2, k0 & 1);
+            pi.pin = k0 & 1;
+        }
+        if (pa.rrow) {  // on this stream too: the adjoint chain is the longer one
+            float* inj = w.inj + set * inj_seg;
+            CK(h, cudaMemsetAsync(inj, 0, (size_t)(k1 - k0) * jb.W * jb.nb * pa.inj_block * 4, su));
+            e = launch_build_injection(jb.rdata, jb.dss, jb.dts, h->nr, k1, k1 - k0, jb.W, jb.nb, h->nuc, h->d_uc_ptr,
+                                       h->d_uc_rec, h->d_uc_pos, inj, pa.inj_block, su);
+            if (e != cudaSuccess) return cuda_fail(h, e, "receiver injection");
+            sw.launches_other++;
+            pa.inj = inj;
+        }
         pi.n0 = k0;
         pi.nsteps = k1 - k0;
         pi.slot0 = set * h->K;
@@ -1022,14 +1049,11 @@ probe_status run_adjoint_res(Sweep& sw, Job& jb, const ResSet& rs) {
         CK(h, cudaEventRecord(h->ov_inc[set], su));
         CK(h, cudaStreamWaitEvent(st, h->ov_inc[set], 0));
         record(h, ev++, st);
-        Sweep one;  // this job's injection
-        one.jobs.push_back(jb);
-        one.st = st;
-        TRY(build_injection(one, k1, k0 + 1));
-        sw.launches_other += one.launches_other;
         pa.n0 = k1;
         pa.nsteps = k1 - k0;
         pa.slot0 = set * h->K + (k1 - k0 - 1);  // level n uses Dtt u^{n-1}
+        pa.pin = (k1 + 1) & 1;
+        pa.pout = (k0 + 1) & 1;
         e = launch_res2d(RES_ADJ, h->kahan != 0, rs.adj, pa, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "adjoint segment launch");
         CK(h, cudaEventRecord(h->ov_born[set], st));

@@ -40,6 +40,17 @@ __device__ __forceinline__ P4 p4add_one(const P4& x, const P4& y, float one) {
     return p4fma(x, p4(one, one, one, one), y);
 }
 
+// 16 bytes from global to shared memory without passing through registers
+__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// The two halves of a cluster barrier that orders no memory
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait;" ::: "memory"); }
+
 struct Strip {  // rows of one CTA
     int z0, rows;
 };
@@ -91,13 +102,38 @@ __global__ void __launch_bounds__(kResThreads, 1) k_res2d(const __grid_constant_
     const bool up = rank > 0, dn = rank < C - 1;
     const long long F = p.F;
     // two levels in shared memory, level k of the launch in the (k & 1)-th: the first to be differentiated at smem
-    const int pl0 = (MODE == RES_ADJ) ? ((p.n0 + 1) & 1) : (p.n0 & 1);
-    float* st0 = p.state + ((long long)unit * 2 + pl0) * F;
-    float* st1 = p.state + ((long long)unit * 2 + (pl0 ^ 1)) * F;
+    const float* in0 = p.in + ((long long)unit * 2 + p.pin) * F;
+    const float* in1 = p.in + ((long long)unit * 2 + (p.pin ^ 1)) * F;
     float* gimg = (MODE == RES_ADJ) ? p.img + (long long)unit * F : nullptr;
     float* gcmp = (MODE == RES_ADJ && KAHAN) ? p.comp + (long long)unit * F : nullptr;
 
-    for (int i = tid; i < 2 * BR * PW / 4; i += nthr) reinterpret_cast<float4*>(smem)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    // Everything the segment reads from memory but Dtt, as asynchronous copies, a warp per row: no
+    // thread waits for a load before it issues its next, and the tables below are made meanwhile.
+    // Cells off the grid are zero in both levels (a neighbour's rows arrive after the cluster barrier).
+    const int warp = tid >> 5, lane = tid & 31, nwarp = nthr >> 5;
+    for (int r = warp; r < BR; r += nwarp) {
+        const int z = z0 - 4 + r;
+        const bool row0 = z >= 0 && z < p.Nz && r < R + 8, row1 = r >= 4 && r < R + 4;
+        for (int g = lane; g < gx + 2; g += 32) {
+            const bool col = g >= 1 && g <= gx;
+            float* lv = smem + r * PW + 4 * g;
+            const long long off = (long long)z * p.P + 4 * (g - 1);
+            if (row0 && col)
+                cp_async16(lv, in0 + off);
+            else
+                st4(lv, make_float4(0.f, 0.f, 0.f, 0.f));
+            if (row1 && col) {
+                const int q = (r - 4) * PX + 4 * (g - 1);
+                cp_async16(lv + BR * PW, in1 + off);
+                cp_async16(S + q, p.s + off);
+                if (MODE == RES_BORN) cp_async16(A1 + q, p.dm + (long long)b * F + off);
+                if (MODE == RES_ADJ) cp_async16(A1 + q, gimg + off);
+                if (MODE == RES_ADJ && KAHAN) cp_async16(A2 + q, gcmp + off);
+            } else {
+                st4(lv + BR * PW, make_float4(0.f, 0.f, 0.f, 0.f));
+            }
+        }
+    }
     for (int i = tid; i < PX; i += nthr) {
         const int rx = max(max(p.pad - i, i - (p.pad + p.nx - 1)), 0);
         xt[i] = __fmul_rn(p.cx, (float)(rx * rx));
@@ -122,20 +158,6 @@ __global__ void __launch_bounds__(kResThreads, 1) k_res2d(const __grid_constant_
         if (C > 1 && p.nsteps >= 2) mbar_arm_tx(&bars[1], rx_bytes);
         if (C > 1 && p.nsteps >= 3) mbar_arm_tx(&bars[0], rx_bytes);
     }
-    __syncthreads();
-    for (int i = tid; i < (R + 8) * gx; i += nthr) {
-        const int r = i / gx, g = i - r * gx, z = z0 - 4 + r;
-        if (z < 0 || z >= p.Nz) continue;
-        const long long off = (long long)z * p.P + 4 * g;
-        st4(smem + r * PW + 4 + 4 * g, ld4(st0 + off));
-        if (r < 4 || r >= R + 4) continue;
-        st4(smem + (BR + r) * PW + 4 + 4 * g, ld4(st1 + off));
-        const int q = (r - 4) * PX + 4 * g;
-        st4(S + q, ld4(p.s + off));
-        if (MODE == RES_BORN) st4(A1 + q, ld4(p.dm + (long long)b * F + off));
-        if (MODE == RES_ADJ) st4(A1 + q, ld4(gimg + off));
-        if (MODE == RES_ADJ && KAHAN) st4(A2 + q, ld4(gcmp + off));
-    }
     uint32_t halo_up = 0, halo_dn = 0, bar_up = 0, bar_dn = 0;  // neighbours' halo rows (of the first level) and bars[0]
     if (up) {
         const int rows_up = strip_of(p.Nz, C, rank - 1).rows;
@@ -146,11 +168,6 @@ __global__ void __launch_bounds__(kResThreads, 1) k_res2d(const __grid_constant_
         halo_dn = mapa_rank(smem_u32(smem + 4), (uint32_t)(rank + 1));
         bar_dn = mapa_rank(smem_u32(&bars[0]), (uint32_t)(rank + 1));
     }
-    if (C > 1)
-        cluster_sync_all();
-    else
-        __syncthreads();
-
     const int nrb = (R + RB - 1) / RB, ntask = nrb * gx;
     const int dq = nthr / gx, dr = nthr - dq * gx;
     const int t0q = tid / gx, t0r = tid - t0q * gx;
@@ -180,6 +197,12 @@ __global__ void __launch_bounds__(kResThreads, 1) k_res2d(const __grid_constant_
                                 : make_float4(0.f, 0.f, 0.f, 0.f);
     };
     if (MODE != RES_INC && tid < ntask) fetch_dtt(0, t0q, t0r, dpre);
+
+    cp_async_wait_all();
+    if (C > 1)
+        cluster_sync_all();
+    else
+        __syncthreads();
 
     for (int k = 0; k < p.nsteps; ++k) {
         const float* cur = smem + (k & 1) * BR * PW;
@@ -317,19 +340,21 @@ __global__ void __launch_bounds__(kResThreads, 1) k_res2d(const __grid_constant_
             break;
         }
     }
+    // No CTA leaves while a neighbour's stores may still be on their way to it.
+    if (C > 1) cluster_arrive_relaxed();
     // both levels back, the image with them
     const float *c0 = smem + (p.nsteps & 1) * BR * PW, *c1 = smem + ((p.nsteps & 1) ^ 1) * BR * PW;
-    float* g0 = (p.nsteps & 1) ? st1 : st0;
-    float* g1 = (p.nsteps & 1) ? st0 : st1;
-    for (int i = tid; i < R * gx; i += nthr) {
-        const int r = i / gx, g = i - r * gx;
-        const long long off = (long long)(z0 + r) * p.P + 4 * g;
-        st4(g0 + off, ld4(c0 + (r + 4) * PW + 4 + 4 * g));
-        st4(g1 + off, ld4(c1 + (r + 4) * PW + 4 + 4 * g));
-        if (MODE == RES_ADJ) st4(gimg + off, ld4(A1 + r * PX + 4 * g));
-        if (MODE == RES_ADJ && KAHAN) st4(gcmp + off, ld4(A2 + r * PX + 4 * g));
-    }
-    if (C > 1) cluster_sync_all();  // no CTA leaves while a neighbour's stores may still be on their way to it
+    for (int r = warp; r < R; r += nwarp)
+        for (int g = lane; g < gx; g += 32) {
+            const long long off = (long long)(z0 + r) * p.P + 4 * g;
+            if (p.out) {
+                st4(p.out + ((long long)unit * 2 + p.pout) * F + off, ld4(c0 + (r + 4) * PW + 4 + 4 * g));
+                st4(p.out + ((long long)unit * 2 + (p.pout ^ 1)) * F + off, ld4(c1 + (r + 4) * PW + 4 + 4 * g));
+            }
+            if (MODE == RES_ADJ) st4(gimg + off, ld4(A1 + r * PX + 4 * g));
+            if (MODE == RES_ADJ && KAHAN) st4(gcmp + off, ld4(A2 + r * PX + 4 * g));
+        }
+    if (C > 1) cluster_wait();
 }
 
 template <int MODE, bool KAHAN, int RB>
