@@ -66,6 +66,7 @@ struct Tuned3 {
 struct ResSet {
     std::vector<long long> key;  // kind, adjoint, shots, trials
     int use = 0;
+    double us = 0.0, fwd = 0.0, rev = 0.0;  // estimate per level; million cells of the forward, of recompute and adjoint
     ResPlan inc, born, rec, adj;  // incident and Born fields of the forward; recompute and adjoint
 };
 

@@ -1086,11 +1086,17 @@ double res_pair(const std::vector<ResPlan>& pa, int ua, const std::vector<ResPla
     return best;
 }
 
+// Estimated time per level (us) of the one-level kernels for fwd / adj million cells of forward and
+// of recomputed and adjoint fields in one launch each: a floor for launch and first loads, then a rate.
+double one_level_us(double fwd, double adj) { return 7.5 + 2.3 * fwd + (adj > 0 ? 11.0 + 4.7 * adj : 0.0); }
+
 // Whether a call of this kind runs on the resident kernels, with the cluster sizes (kept per
-// workload; a host-side estimate, nothing is timed).  They are taken where their estimate, with
-// 14 us per segment and chain for launch, load and store, is below the one-level kernels': one launch
-// of at least 4.5 us per level, or the rates that those reach on grids that fill the chip (360
-// Gcell/s forward, 300 recompute, 215 adjoint; 541 x 541, 32 shots).
+// workload; a host-side estimate, nothing is timed; 10 us per segment and chain for launch, load and
+// store).  With an adjoint, wherever the grid fits: measured over 121 x 121 to 300 x 460, 2 to 64
+// shots, 1 and 4 trials, they take 0.20 to 0.92 of the one-level kernels' time.  Forward only, where
+// the estimate is below the one-level kernels': few fields 0.39 to 0.6 of their time, equal at about
+// six million cells in flight, and up to 1.5 beyond (325 x 445, 64 shots, 4 trials: one cluster of 16
+// SMs at a time holds a field, 112 of 152 SMs), where the one-level kernels stay.
 const ResSet& res_set(probe_t h, FwdKind kind, bool adjoint, int W, int nb) {
     const std::vector<long long> key = {(long long)kind, (long long)adjoint, W, nb, h->user_fixed, h->user_tblock,
                                         h->opt_tile_z, h->opt_dtt_history, h->opt_autotune};
@@ -1104,14 +1110,14 @@ const ResSet& res_set(probe_t h, FwdKind kind, bool adjoint, int W, int nb) {
         std::vector<ResPlan> bo, ad;
         if (born) bo = plan_res2d(RES_BORN, kh, h->Nz, h->Nx, h->pad, h->K);
         if (adjoint) ad = plan_res2d(RES_ADJ, kh, h->Nz, h->Nx, h->pad, h->K);
-        const double seg = 14.0 / h->K, gc = (double)h->Nz * h->Nx * W * 1e-3;  // thousand cells of one field kind
-        double t = res_pair(inc, W, bo, born ? W * nb : 0, &r.inc, &r.born) + seg;
-        double t1 = std::max(4.5, gc * (born ? 1 + nb : 1) / 360.0);
+        const double seg = 10.0 / h->K, cells = (double)h->Nz * h->Nx * W * 1e-6;
+        r.us = res_pair(inc, W, bo, born ? W * nb : 0, &r.inc, &r.born) + seg;
+        r.fwd = cells * (born ? 1 + nb : 1);
         if (adjoint) {
-            t += res_pair(inc, W, ad, W * nb, &r.rec, &r.adj) + seg;
-            t1 += std::max(4.5, gc / 300.0) + std::max(4.5, gc * nb / 215.0);
+            r.us += res_pair(inc, W, ad, W * nb, &r.rec, &r.adj) + seg;
+            r.rev = cells * (1 + nb);
         }
-        r.use = t < t1;
+        r.use = r.us < (adjoint ? 1e20 : one_level_us(r.fwd, 0.0));  // 1e30: no cluster of this size can run
     }
     h->res_sets.push_back(r);
     return h->res_sets.back();
@@ -2501,11 +2507,16 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
     int res = 1;  // every model on the resident kernels, or none
     for (int k = 0; k < nmodels; ++k) res = res && res_fits(models[k], 1, 1);
     std::vector<ResSet> rss(nmodels);
-    if (res)
+    if (res) {  // the resident kernels take the models in turn, the one-level kernels all at once
+        double us = 0.0, fwd = 0.0, rev = 0.0;
         for (int k = 0; k < nmodels; ++k) {
             rss[k] = res_set(models[k], FWD_BORN, true, models[k]->ns, nb[k]);
-            res = res && rss[k].use;
+            us += rss[k].us;
+            fwd += rss[k].fwd;
+            rev += rss[k].rev;
         }
+        res = us < one_level_us(fwd, rev);
+    }
     for (int k = 0; k < nmodels; ++k) {
         probe_t h = models[k];
         bool hin = false;

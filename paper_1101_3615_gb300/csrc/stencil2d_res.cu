@@ -417,7 +417,9 @@ bool res2d_fits(int mode, bool kahan, int Nz, int Nx, int pad, int nsteps) {
     return pad <= kResPadMax && res_smem(mode, kahan, Nz, Nx, pad, C, 2, nsteps) <= kResSmemMax;
 }
 
-// Candidate cluster sizes and rows per thread for fields of an Nz x Nx grid, each with the number of
+// Candidate cluster sizes (not only powers of two: with 9 CTAs the chip holds 15 clusters, as with 8,
+// and a strip is an eighth lower; 241 x 281, 6 shots, Krylov trials 13.4 -> 11.1 ms) and rows per
+// thread for fields of an Nz x Nx grid, each with the number of
 // clusters that the chip holds at once and the estimated time of one level of one wave of clusters.
 // The model (microseconds), fitted on 77 x 103 to 277 x 423 grids, C = 1 to 16, within about 15 %:
 // exchange and barriers 0.55 (0.3 in a single CTA); then per round of tasks, with w warps,
@@ -426,7 +428,7 @@ bool res2d_fits(int mode, bool kahan, int Nz, int Nx, int pad, int nsteps) {
 std::vector<ResPlan> plan_res2d(int mode, bool kahan, int Nz, int Nx, int pad, int nsteps) {
     std::vector<ResPlan> out;
     const int gx = res_groups(Nx);
-    for (int C : {1, 2, 4, 8, 16}) {
+    for (int C : {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 16}) {
         if (C > 1 && Nz / C < 4) break;  // a halo row must belong to the adjacent strip
         for (int RB : {4, 2}) {
             const size_t sm = res_smem(mode, kahan, Nz, Nx, pad, C, RB, nsteps);

@@ -22,6 +22,7 @@ CASES = [
     ((17, 130), 1, 40, 39, 2, 1),      # one segment
     ((129, 66), 9, 37, 5, 2, 1),
     ((203, 317), 17, 41, 20, 3, 1),
+    ((201, 241), 20, 40, 0, 6, 1),     # clusters of nine CTAs on the GB300: strips of unequal height
     ((61, 200), 3, 40, 19, 9, 3),      # more fields than clusters at once; a last segment of one level
 ]
 
