@@ -186,22 +186,31 @@ long long inj_block(probe_t h) { return (long long)h->nband * (h->ndim == 3 ? (l
 // Bytes per resident shot and fixed bytes of a job with nb trials.
 bool use_history(probe_t h, int with_ckpt) { return with_ckpt && h->opt_dtt_history && h->ndim == 2; }
 
+// Levels of one launch of the resident kernels.  A call with checkpoints: the checkpoint stride.
+// Without: twice that (a launch costs about 6 us, a level of the smallest grids 0.9, and the Born chain
+// starts one segment late: 77 x 103, nt = 200, 15 -> 30 levels: 430 -> 396 us), as long as the Dtt
+// planes of two segments stay in L2.
+int res_seg(probe_t h, int with_ckpt) {
+    const bool longer = !with_ckpt && 16.0 * h->K * h->ns * h->F <= 48e6;
+    return std::min(h->nt - 1, (longer ? 2 : 1) * h->K);
+}
+
 // 2D calls may run on the cluster-resident kernels (stencil2d_res.cu): no kernel variant or Dtt
 // history chosen by the caller, and a strip of at least four rows of some cluster's CTA holds the
 // two levels and the pointwise operands of the fields that the call advances.
 bool res_fits(probe_t h, int with_ckpt, int born) {
     if (h->ndim != 2 || h->user_fixed || h->user_tblock || h->opt_tile_z || h->opt_dtt_history || !h->opt_autotune)
         return false;
-    const bool kh = h->kahan != 0;
-    return res2d_fits(RES_INC, kh, h->Nz, h->Nx, h->pad, h->K) && (!born || res2d_fits(RES_BORN, kh, h->Nz, h->Nx, h->pad, h->K)) &&
-           (!with_ckpt || res2d_fits(RES_ADJ, kh, h->Nz, h->Nx, h->pad, h->K));
+    const int T = res_seg(h, with_ckpt);
+    auto fits = [&](int mode) { return res2d_fits(mode, h->kahan != 0, h->Nz, h->Nx, h->pad, T); };
+    return fits(RES_INC) && (!born || fits(RES_BORN)) && (!with_ckpt || fits(RES_ADJ));
 }
 
-// Dtt planes per shot of a 2D workspace: the history; two checkpoint segments for the resident
-// kernels (one being read while the next is written); one segment; none (1, unallocated).
+// Dtt planes per shot of a 2D workspace: the history; two segments for the resident kernels (one
+// being read while the next is written); one checkpoint segment; none (1, unallocated).
 int dtt_slots_2d(probe_t h, int with_ckpt, int history, int res) {
     if (history) return h->nt - 1;
-    if (res) return 2 * h->K;
+    if (res) return 2 * res_seg(h, with_ckpt);
     return with_ckpt ? h->K : 1;
 }
 
@@ -220,7 +229,7 @@ void ws_bytes(probe_t h, int nb, int with_ckpt, int with_data, int res, double* 
     else if (h->ndim == 3)
         ps += 2.0 * F4;  // Dtt u^n of two steps (Born source)
     else if (res)
-        ps += 2.0 * h->K * F4;
+        ps += 2.0 * res_seg(h, 0) * F4;
     if (with_data) ps += (double)nb * h->nt * h->nr * 4.0;
     if (h->ndim == 3 && with_ckpt) {
         ps += 2.0 * nb * F4;  // per-shot images + compensation
@@ -283,7 +292,8 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, i
     const int G = W;  // image groups for the smallest shot group: any group size fits
     const int history = use_history(h, with_ckpt) ? 1 : 0;
     const int slots2 = h->ndim == 2 ? dtt_slots_2d(h, with_ckpt, history, res) : 0;
-    if (w.u && (h->ndim == 3 || w.dtt_slots >= slots2) && w.W >= W && w.nb >= nb && w.with_ckpt >= with_ckpt && w.with_data >= with_data &&
+    // (a workspace with checkpoint segments serves calls without them, in shorter launches)
+    if (w.u && (h->ndim == 3 || w.dtt_slots >= std::min(slots2, 2 * h->K)) && w.W >= W && w.nb >= nb && w.with_ckpt >= with_ckpt && w.with_data >= with_data &&
         w.groups >= G && w.tm_tile_z == h->tile_z && w.W == W && w.nb == nb && w.history == history)
         return PROBE_OK;
     free_ws(w);
@@ -950,8 +960,9 @@ probe_status run_forward_res(Sweep& sw, Job& jb, const ResSet& rs, FwdKind kind,
         CK(h, cudaEventRecord(h->ov_inc[0], st));
         CK(h, cudaStreamWaitEvent(su, h->ov_inc[0], 0));
     }
-    for (int n = 0, i = 0; n < h->nt - 1; n += h->K, ++i) {
-        const int T = std::min(h->K, h->nt - 1 - n), set = i & 1;
+    const int seg = born ? std::min(res_seg(h, ckpt), w.dtt_slots / 2) : res_seg(h, ckpt);
+    for (int n = 0, i = 0; n < h->nt - 1; n += seg, ++i) {
+        const int T = std::min(seg, h->nt - 1 - n), set = i & 1;
         if (born && i >= 2) CK(h, cudaStreamWaitEvent(su, h->ov_born[set], 0));
         pi.pin = pb.pin = n & 1;
         pi.pout = pb.pout = (n + T) & 1;
@@ -967,7 +978,7 @@ probe_status run_forward_res(Sweep& sw, Job& jb, const ResSet& rs, FwdKind kind,
         }
         pi.n0 = pb.n0 = n;
         pi.nsteps = pb.nsteps = T;
-        pi.slot0 = pb.slot0 = set * h->K;
+        pi.slot0 = pb.slot0 = set * seg;
         pi.dtt = born ? w.dtt : nullptr;
         cudaError_t e = launch_res2d(RES_INC, false, rs.inc, pi, su);
         if (e != cudaSuccess) return cuda_fail(h, e, "incident segment launch");
@@ -1106,11 +1117,12 @@ const ResSet& res_set(probe_t h, FwdKind kind, bool adjoint, int W, int nb) {
     r.key = key;
     const bool born = kind == FWD_BORN, kh = h->kahan != 0;
     if (res_fits(h, adjoint, born)) {
-        const std::vector<ResPlan> inc = plan_res2d(RES_INC, kh, h->Nz, h->Nx, h->pad, h->K);
+        const int T = res_seg(h, adjoint);
+        const std::vector<ResPlan> inc = plan_res2d(RES_INC, kh, h->Nz, h->Nx, h->pad, T);
         std::vector<ResPlan> bo, ad;
-        if (born) bo = plan_res2d(RES_BORN, kh, h->Nz, h->Nx, h->pad, h->K);
-        if (adjoint) ad = plan_res2d(RES_ADJ, kh, h->Nz, h->Nx, h->pad, h->K);
-        const double seg = 10.0 / h->K, cells = (double)h->Nz * h->Nx * W * 1e-6;
+        if (born) bo = plan_res2d(RES_BORN, kh, h->Nz, h->Nx, h->pad, T);
+        if (adjoint) ad = plan_res2d(RES_ADJ, kh, h->Nz, h->Nx, h->pad, T);
+        const double seg = 10.0 / T, cells = (double)h->Nz * h->Nx * W * 1e-6;
         r.us = res_pair(inc, W, bo, born ? W * nb : 0, &r.inc, &r.born) + seg;
         r.fwd = cells * (born ? 1 + nb : 1);
         if (adjoint) {
@@ -2205,7 +2217,7 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
             }
             h->stats.pipeline_rows = piped ? h->ws_rows : 0;
             h->stats.pipeline_rows_adjoint = piped ? h->ws_rows_adj : 0;
-            h->stats.time_block = rs.use ? h->K : (h->ndim == 2 && h->tile_z == kPipeTZ && w.u4) ? h->opt_tblock : 1;
+            h->stats.time_block = rs.use ? res_seg(h, need_ckpt) : (h->ndim == 2 && h->tile_z == kPipeTZ && w.u4) ? h->opt_tblock : 1;
             if (need_ckpt) {
                 CK(h, cudaMemsetAsync(w.img, 0, (size_t)G * nbw * h->F * 4, st));
                 CK(h, cudaMemsetAsync(w.comp, 0, (size_t)G * nbw * h->F * 4, st));

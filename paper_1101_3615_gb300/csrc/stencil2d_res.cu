@@ -357,11 +357,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_res2d(const __grid_constant_
     if (C > 1) cluster_wait();
 }
 
-template <int MODE, bool KAHAN, int RB>
-cudaError_t res_config(int C, int threads, size_t smem, int units, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr) {
-    auto kernel = k_res2d<MODE, KAHAN, RB>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+void res_config(int C, int threads, size_t smem, int units, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr) {
     cfg = {};
     cfg.gridDim = dim3((unsigned)(C * units));
     cfg.blockDim = dim3((unsigned)threads);
@@ -372,31 +368,33 @@ cudaError_t res_config(int C, int threads, size_t smem, int units, cudaLaunchCon
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return e;
+}
+
+// A plan is made before its first launch, so the kernel's limits (raised to the most that any plan
+// uses) are set here and not with each launch.
+template <int MODE, bool KAHAN, int RB>
+int res_clusters(int C, int threads, size_t smem) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    res_config(C, threads, smem, 1, cfg, attr);
+    int n = 0;
+    auto kernel = k_res2d<MODE, KAHAN, RB>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmemMax) != cudaSuccess ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n;
 }
 
 template <int MODE, bool KAHAN, int RB>
 cudaError_t res_launch(const ResPlan& pl, const ResParams2D& p, int units, cudaStream_t st) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    cudaError_t e = res_config<MODE, KAHAN, RB>(pl.C, pl.threads, res_smem(MODE, KAHAN, p.Nz, p.Nx, p.pad, pl.C, RB, p.nsteps),
-                                                units, cfg, attr);
-    if (e != cudaSuccess) return e;
+    res_config(pl.C, pl.threads, res_smem(MODE, KAHAN, p.Nz, p.Nx, p.pad, pl.C, RB, p.nsteps), units, cfg, attr);
     cfg.stream = st;
     return cudaLaunchKernelEx(&cfg, k_res2d<MODE, KAHAN, RB>, p);
-}
-
-template <int MODE, bool KAHAN, int RB>
-int res_clusters(int C, int threads, size_t smem) {
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[1];
-    int n = 0;
-    if (res_config<MODE, KAHAN, RB>(C, threads, smem, 1, cfg, attr) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, k_res2d<MODE, KAHAN, RB>, &cfg) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return n;
 }
 
 template <int MODE, bool KAHAN>
