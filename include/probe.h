@@ -247,7 +247,8 @@ probe_status probe_apply_H_group(const probe_t* models, int nmodels,
  * (the least-squares problem whose normal equations M c = (Bx)^T y,
  * M_ik = sum_j (B_i x_j)^T (B_k x_j), Sec. 1.4 writes).  Solved on the device
  * in FP64 through a QR factorisation of the stacked columns A = [B_i x_j]
- * (CholeskyQR2: Cholesky QR with one reorthogonalisation), so the error grows
+ * (Cholesky QR with one refinement step, or with one reorthogonalisation,
+ * CholeskyQR2, where cond(A) is above about 1e4), so the error grows
  * like cond(A) eps, not cond(A)^2 eps.  coeffs (host or device) and resid_rel
  * (||y - Bx c|| / ||y||, host) are written; the call synchronises.
  * Returns PROBE_ERR_STATE if the columns are numerically rank deficient. */

@@ -55,6 +55,35 @@ def test_fit_gram_paths_match_oracle(cuda_device, shape, spatial, angular, nradi
     assert abs(res - res_orc) < 1e-7
 
 
+@pytest.mark.parametrize("spatial,angular,nradial,sigma", [
+    (MODES2[16:32], [0, 2], 2, 0),          # P = 64, cond 9: refined
+    (MODES2[:3], [0, 2, -2, 4], 3, 2),      # cond 1e2
+    ([(0, 0)], [0, 2], 7, 0),               # cond 4e2, one spatial mode
+    ([(0, 0), (1, 0)], [0, 2], 8, 3),       # cond 2e5: the reorthogonalising pass
+    ([(0, 0), (1, 0)], [0, 2], 10, 3),      # cond 1e6
+    ([(0, 0)], [0, 2], 14, 3),              # cond 2e7
+])
+def test_fit_refinement_has_the_accuracy_of_qr(cuda_device, spatial, angular, nradial, sigma):
+    """Targets that the basis cannot fit (residual of the size of the target) and columns of growing
+    condition number: the coefficients against Householder QR within the perturbation bound of the
+    least-squares problem, eps cond (2 + cond |r| / (|A| |c|)) with eps = 1e-14 (columns from another FFT)."""
+    from scipy.ndimage import gaussian_filter
+    shape = (43, 51)
+    wl, probe, g, o = setup(shape, spatial, angular, nradial, -1.0, 5)
+    xs = np.random.default_rng(4).standard_normal((2,) + shape)
+    if sigma:
+        xs = np.stack([gaussian_filter(x, sigma) for x in xs])
+    xs = xs.astype(np.float32)
+    A = np.concatenate([o.columns(x.astype(np.float64)) for x in xs])
+    ys = (np.random.default_rng(5).standard_normal((2,) + shape) * np.linalg.norm(A, axis=1).mean()).astype(np.float32)
+    c_orc, res_orc, cond = ofit(o, ys, xs)
+    c, res = probe.fit(g, torch.tensor(ys, device=cuda_device), torch.tensor(xs, device=cuda_device))
+    r = res_orc * np.linalg.norm(ys.astype(np.float64))
+    bound = 1e-14 * cond * (2 + cond * r / (np.linalg.norm(A, 2) * np.linalg.norm(c_orc)))
+    assert rel(c, c_orc) < bound, (cond, bound)
+    assert abs(res - res_orc) < 1e-12
+
+
 @pytest.mark.parametrize("order", [-1.0, 0.0, 0.5])
 @pytest.mark.parametrize("shape,spatial,angular,nradial", [
     ((33, 40), MODES2[:6], [0, 2, -2, 7, -5], 5),
