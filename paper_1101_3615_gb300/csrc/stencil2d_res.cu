@@ -399,11 +399,13 @@ cudaError_t res_launch(const ResPlan& pl, const ResParams2D& p, int units, cudaS
 
 template <int MODE, bool KAHAN>
 int res_clusters_rb(int RB, int C, int threads, size_t smem) {
+    if (RB == 1) return res_clusters<MODE, KAHAN, 1>(C, threads, smem);
     return RB == 4 ? res_clusters<MODE, KAHAN, 4>(C, threads, smem) : res_clusters<MODE, KAHAN, 2>(C, threads, smem);
 }
 
 template <int MODE, bool KAHAN>
 cudaError_t res_launch_rb(const ResPlan& pl, const ResParams2D& p, int units, cudaStream_t st) {
+    if (pl.RB == 1) return res_launch<MODE, KAHAN, 1>(pl, p, units, st);
     return pl.RB == 4 ? res_launch<MODE, KAHAN, 4>(pl, p, units, st) : res_launch<MODE, KAHAN, 2>(pl, p, units, st);
 }
 
@@ -421,14 +423,16 @@ bool res2d_fits(int mode, bool kahan, int Nz, int Nx, int pad, int nsteps) {
 // clusters that the chip holds at once and the estimated time of one level of one wave of clusters.
 // The model (microseconds), fitted on 77 x 103 to 277 x 423 grids, C = 1 to 16, within about 15 %:
 // exchange and barriers 0.55 (0.3 in a single CTA); then per round of tasks, with w warps,
-// max(0.73, 0.45 + 0.078 w) with four rows per thread, max(0.32, 0.2 + 0.045 w) with two; Born 1.17,
-// adjoint 1.4 times that.
+// max(0.73, 0.45 + 0.078 w) with four rows per thread, max(0.32, 0.2 + 0.045 w) with two,
+// max(0.22, 0.1 + 0.034 w) with one; Born 1.17, adjoint 1.4 times that.  More rows per thread share more
+// differences, fewer make a shorter chain: 77 x 103, clusters of 16, a level of the incident field
+// 1.24, 0.93 and 0.79 us with four, two and one; 241 x 281 1.65, 1.89 and 1.85.
 std::vector<ResPlan> plan_res2d(int mode, bool kahan, int Nz, int Nx, int pad, int nsteps) {
     std::vector<ResPlan> out;
     const int gx = res_groups(Nx);
     for (int C : {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 12, 14, 16}) {
         if (C > 1 && Nz / C < 4) break;  // a halo row must belong to the adjacent strip
-        for (int RB : {4, 2}) {
+        for (int RB : {4, 2, 1}) {
             const size_t sm = res_smem(mode, kahan, Nz, Nx, pad, C, RB, nsteps);
             if (sm > kResSmemMax) continue;
             const int rows = (Nz + C - 1) / C, ntask = (rows + RB - 1) / RB * gx;
@@ -446,8 +450,10 @@ std::vector<ResPlan> plan_res2d(int mode, bool kahan, int Nz, int Nx, int pad, i
             }
             if (pl.clusters < 1) continue;
             const double f = mode == RES_INC ? 1.0 : (mode == RES_BORN ? 1.17 : 1.4), w = pl.threads / 32;
-            pl.us = (C > 1 ? 0.55 : 0.3) +
-                    f * rounds * (RB == 4 ? std::max(0.73, 0.45 + 0.078 * w) : std::max(0.32, 0.2 + 0.045 * w));
+            const double task = RB == 4   ? std::max(0.73, 0.45 + 0.078 * w)
+                                : RB == 2 ? std::max(0.32, 0.2 + 0.045 * w)
+                                          : std::max(0.22, 0.1 + 0.034 * w);
+            pl.us = (C > 1 ? 0.55 : 0.3) + f * rounds * task;
             out.push_back(pl);
         }
     }
