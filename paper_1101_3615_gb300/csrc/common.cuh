@@ -132,7 +132,8 @@ __device__ __forceinline__ void cluster_sync_all() {
 // Rounding-explicit pieces of the explicit time update u^{n+1} = G (2 u^n - a- u^{n-1} + rhs)
 // (Sec. 2 scheme with the sponge).  Every product and sum is one IEEE operation written
 // out, so the compiler cannot fuse them differently in different kernel instantiations:
-// all 2D variants (one tile per CTA, pipelined, single- or multi-model) give the same bits.
+// the 2D variants give the same bits (the pipelined kernels' packed all-interior path excepted, where
+// the compiler fuses a product and a sum).
 __device__ __forceinline__ float leapfrog(float G, float c, float am, float prev, float rhs) {
     return __fmul_rn(G, __fadd_rn(__fmaf_rn(-am, prev, __fadd_rn(c, c)), rhs));
 }
