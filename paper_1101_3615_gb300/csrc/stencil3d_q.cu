@@ -13,6 +13,13 @@
 //     holds mu^{n+1} (the differentiated level) and mu^{n+2} (the level it overwrites), so it adds the
 //     imaging terms of all three, in the order in which the single steps would.
 //
+// What bounds it: issue and operand latency at two CTAs (18 warps) per SM below DRAM -- 300 instructions
+// per warp and plane, issue active half of the cycles, DRAM 5.1 to 5.8 TB/s in the adjoint and 4.2 in
+// the incident step (168 x 256 x 296, 4 shots, 4 trials).  Measured against the kernels of
+// stencil3d.cu as they were tuned, whole calls: H on 296^3 (padded), 8 shots, 4 trials, 60 levels 528 ->
+// 465 ms; H on 116 x 101 x 141, 3 shots 45.2 -> 34.7 ms; F on 168^3, 4 shots, 2 trials 42.9 -> 38.8 ms.
+// Slower variants: two trials per CTA, two rows per thread, a refill by the last compute warp.
+//
 // The per-cell arithmetic is that of cells3 in stencil3d.cu, operation for operation: same bits.
 #include "common.cuh"
 #include "internal.h"
