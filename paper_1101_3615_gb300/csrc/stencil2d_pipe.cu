@@ -378,10 +378,13 @@ __global__ void __launch_bounds__(kWsThreads, R == 1 ? 4 : 3) k_fwd2d_ws(const _
 // of one row per thread sit on an SM, instead of 2, and takes the z taps in packed FP32x2.  us per
 // time step, before -> after: 32 shots of 541^2, one trial 43.3 -> 40.9; gradient, 8 shots of 1041^2
 // 37.3 -> 35.3; group of 341^2, 541^2 and 741^2, 8 shots x 4 trials each 158 -> 144.
-constexpr int adj_ctas(int nbc, int r) { return nbc * r >= 8 ? 1 : r == 2 ? 2 : nbc == 1 ? 4 : 3; }
+// With fewer than three items for each of those CTAs a CTA has too little to pipeline, and the variant
+// of two CTAs per SM stays (MANY = false): Krylov chains on 238 x 584 (9 shots) and 548 x 454 (4 shots)
+// ran 1.2 and 1.1 % slower with four.
+constexpr int adj_ctas(int nbc, int r, bool many) { return nbc * r >= 8 ? 1 : r == 2 || !many ? 2 : nbc == 1 ? 4 : 3; }
 
-template <int NBC, bool KAHAN, int S, bool MULTI, int R>
-__global__ void __launch_bounds__(kWsThreads, adj_ctas(NBC, R)) k_adj2d_ws(const __grid_constant__ StepParams2D p) {
+template <int NBC, bool KAHAN, int S, bool MULTI, int R, bool MANY>
+__global__ void __launch_bounds__(kWsThreads, adj_ctas(NBC, R, MANY)) k_adj2d_ws(const __grid_constant__ StepParams2D p) {
     using T = Ws<R>;
     extern __shared__ __align__(128) float smem[];
     __shared__ __align__(8) uint64_t full[S], empty[S];
@@ -616,15 +619,23 @@ cudaError_t launch_fwd_kr(int stages, const StepParams2D& p, cudaStream_t st) {
                        : launch_persistent(k_fwd2d_ws<K, 2, false, R>, sm, total, p, st);
 }
 
-template <int NB, bool KH, int R>
-cudaError_t launch_adj_nkr(int stages, const StepParams2D& q, cudaStream_t st) {
+template <int NB, bool KH, int R, bool MANY>
+cudaError_t launch_adj_nkrm(int stages, const StepParams2D& q, cudaStream_t st) {
     const size_t sm = smem_bytes<R>(stages, true);
     const int total = q.total_items;
     if (q.nmodels > 1)
-        return stages == 3 ? launch_persistent(k_adj2d_ws<NB, KH, 3, true, R>, sm, total, q, st)
-                           : launch_persistent(k_adj2d_ws<NB, KH, 2, true, R>, sm, total, q, st);
-    return stages == 3 ? launch_persistent(k_adj2d_ws<NB, KH, 3, false, R>, sm, total, q, st)
-                       : launch_persistent(k_adj2d_ws<NB, KH, 2, false, R>, sm, total, q, st);
+        return stages == 3 ? launch_persistent(k_adj2d_ws<NB, KH, 3, true, R, MANY>, sm, total, q, st)
+                           : launch_persistent(k_adj2d_ws<NB, KH, 2, true, R, MANY>, sm, total, q, st);
+    return stages == 3 ? launch_persistent(k_adj2d_ws<NB, KH, 3, false, R, MANY>, sm, total, q, st)
+                       : launch_persistent(k_adj2d_ws<NB, KH, 2, false, R, MANY>, sm, total, q, st);
+}
+
+template <int NB, bool KH, int R>
+cudaError_t launch_adj_nkr(int stages, const StepParams2D& q, cudaStream_t st) {
+    constexpr int ctas = adj_ctas(NB, R, true);
+    if constexpr (ctas > 2)
+        if (q.total_items >= 3 * num_sms() * ctas) return launch_adj_nkrm<NB, KH, R, true>(stages, q, st);
+    return launch_adj_nkrm<NB, KH, R, false>(stages, q, st);
 }
 
 template <int NB, bool KH>
