@@ -147,11 +147,13 @@ __device__ __forceinline__ KBin kbin(const BasisDev& B, long long r) {
 }
 
 // Angular factor.  2D: cos(q theta), sin(|q| theta) with e^{i theta} = ux + i uz, as the |q|-th
-// power of that unit number by repeated squaring (no inverse or direct trigonometric function).
+// power of that unit number by repeated squaring (no inverse or direct trigonometric function).  |q| as an
+// unsigned number: every index is accepted, and the magnitude of the lowest is no int (as a negative
+// one, shifted right, it would never reach zero).
 __device__ __forceinline__ double angular_factor(const BasisDev& B, const KBin& k, int ang) {
     if (B.ndim == 2) {
         double c = 1.0, s = 0.0, bc = k.ux, bs = k.uz;
-        for (int e = abs(ang); e; e >>= 1) {
+        for (unsigned e = ang < 0 ? 0u - (unsigned)ang : (unsigned)ang; e; e >>= 1) {
             if (e & 1) {
                 const double t = c * bc - s * bs;
                 s = c * bs + s * bc;

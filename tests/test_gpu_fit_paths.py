@@ -97,3 +97,14 @@ def test_precond_spectra_match_oracle(cuda_device, shape, spatial, angular, nrad
     img = np.random.default_rng(9).standard_normal(shape).astype(np.float32)
     got = probe.apply_precond(g, c, torch.tensor(img, device=cuda_device)).cpu().numpy()
     assert rel(got, o.apply(c, img.astype(np.float64))) < 1e-6
+
+
+@pytest.mark.parametrize("q", [2**31 - 1, -2**31 + 1, -2**31])
+def test_angular_indices_at_the_ends_of_their_type(cuda_device, q):
+    """2D angular indices are not bounded.  The angle of a bin is known to 2**-52 of itself, so its multiple by
+    2**31 to about 1e-6; twenty times that for the roundings of 31 squarings and of the oracle's product."""
+    wl, probe, g, o = setup((33, 40), [(0, 0)], [q], 2, -1.0, 3)
+    c = np.random.default_rng(8).standard_normal(g.P)
+    img = np.random.default_rng(9).standard_normal((33, 40)).astype(np.float32)
+    got = probe.apply_precond(g, c, torch.tensor(img, device=cuda_device)).cpu().numpy()
+    assert rel(got, o.apply(c, img.astype(np.float64))) < 2e-5
