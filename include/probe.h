@@ -249,7 +249,7 @@ probe_status probe_apply_H_group(const probe_t* models, int nmodels,
  * M_ik = sum_j (B_i x_j)^T (B_k x_j), Sec. 1.4 writes).  Solved on the device
  * in FP64 through a QR factorisation of the stacked columns A = [B_i x_j]
  * (Cholesky QR with one refinement step, or with one reorthogonalisation,
- * CholeskyQR2, where cond(A) is above about 1e4), so the error grows
+ * CholeskyQR2, where cond(A) is above about 1e4 to 1e5), so the error grows
  * like cond(A) eps, not cond(A)^2 eps.  coeffs (host or device) and resid_rel
  * (||y - Bx c|| / ||y||, host) are written; the call synchronises.
  * Returns PROBE_ERR_STATE if the columns are numerically rank deficient. */

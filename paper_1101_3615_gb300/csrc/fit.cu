@@ -11,15 +11,15 @@
 //     pass 1:  A^T A = R1^T R1                       (Cholesky)
 //     pass 2:  Q1 = A R1^{-1} row by row, Q1^T Q1 = R2^T R2, z = Q1^T y
 //     A = Q R with Q = Q1 R2^{-1}, R = R2 R1:  c = R^{-1} Q^T y = R1^{-1} R2^{-1} R2^{-T} z.
-// Up to 64 terms and cond(A) of about 1e4, pass 2 is replaced by one step of iterative refinement with
-// R1 (fit_refine), a pass over the data at a twentieth of its cost: 128^3, 60 terms, 4 pairs 93 -> 39.8 ms.
+// Up to 64 terms and cond(A) of about 1e5 (1e4 for targets far outside the range of A), pass 2 is replaced by one
+// step of iterative refinement with R1 (fit_refine), a pass over the data at a twentieth of its cost: 128^3, 60 terms, 4 pairs 93 -> 39.8 ms.
 // The Gram matrix of the reorthogonalised Q1 is within a few units of round-off
 // of the identity whenever cond(A) is below about 1e7, so the solution has the
 // accuracy of a Householder QR (error ~ cond(A) eps) instead of the
 // cond(A)^2 eps of the normal equations M c = A^T y that Sec. 1.4 writes; the
 // first Cholesky factorisation fails (PROBE_ERR_STATE) only when A is
 // numerically rank deficient.  Gram matrices: P <= 64 -- pass 1 from the sums over the trials at each
-// point (k_fit_gram_s), pass 2 (above cond 1e4) with the columns formed and solved against R1 in shared memory, one row
+// point (k_fit_gram_s), pass 2 (above those conditions) with the columns formed and solved against R1 in shared memory, one row
 // per thread (k_fit_gram<true>); P up to 1024 -- [A | y] formed in column-major chunks
 // of about 256 MB, R1^{-1} applied row by row, and a tiled FP64 Gram kernel.
 // A second pass forms ||y - sum_i c_i B_i x|| / ||y||.
@@ -812,10 +812,12 @@ __global__ void __launch_bounds__(256) k_fit_refine(const double* __restrict__ w
 }
 
 // One CTA: g = the sum of nblocks partials (P <= 64 each), v = L^{-1} g, coef += L^{-T} v, *norm2 = |v|^2.
-// Each substitution is one warp's, the unknowns in its registers.
+// Each substitution is one warp's, the unknowns in its registers.  With inv2, warps 2 and 3 meanwhile invert
+// L by columns, a column per thread, into the unused half of the staged factor (128^3, P = 60, 4 pairs: no
+// difference in the call's 39.8 ms), and inv2[0] + inv2[1] = |L^{-1} D|_F^2, D = diag of L's row norms (the norms of A's columns).
 __global__ void __launch_bounds__(256) k_fit_refine_step(const double* __restrict__ partial, int nblocks, int P,
                                                          const double* __restrict__ L, double* __restrict__ coef,
-                                                         double* __restrict__ norm2) {
+                                                         double* __restrict__ norm2, double* __restrict__ inv2) {
     __shared__ double Ls[kMaxSmall][kMaxSmall + 1], sums[4][kMaxSmall];
     const int tid = threadIdx.x, lane = tid & 31;
     for (int i = tid; i < P * P; i += 256) Ls[i / P][i % P] = L[i];
@@ -825,6 +827,27 @@ __global__ void __launch_bounds__(256) k_fit_refine_step(const double* __restric
         for (int b = quarter; b < nblocks; b += 4) s += partial[(long long)b * P + t];
     sums[quarter][t] = s;
     __syncthreads();
+    if (inv2 && tid >= 64 && tid < 128) {  // entry (r, t) of the inverse, r >= t, at Ls[t][r + 1]
+        double d2 = 0.0, x2 = 0.0;
+        if (t < P) {
+            for (int k = 0; k <= t; ++k) d2 = fma(Ls[t][k], Ls[t][k], d2);
+            for (int r = t; r < P; ++r) {
+                double v0 = r == t ? 1.0 : 0.0, v1 = 0.0;
+                int k = t;
+                for (; k + 1 < r; k += 2) {
+                    v0 = fma(-Ls[r][k], Ls[t][k + 1], v0);
+                    v1 = fma(-Ls[r][k + 1], Ls[t][k + 2], v1);
+                }
+                if (k < r) v0 = fma(-Ls[r][k], Ls[t][k + 1], v0);
+                const double x = (v0 + v1) / Ls[r][r];
+                Ls[t][r + 1] = x;
+                x2 = fma(x, x, x2);
+            }
+        }
+        double v = d2 * x2;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) inv2[(tid >> 5) - 2] = v;
+    }
     if (tid >= 32) return;
     const int t1 = lane + 32;
     double x0 = (sums[0][lane] + sums[1][lane]) + (sums[2][lane] + sums[3][lane]);
@@ -1095,32 +1118,39 @@ probe_status fit_cholesky(probe_t h, double* C, int n, int P, double* L, double*
 // Least squares with the factor of the first pass alone (P <= 64): c = (L1 L1^T)^{-1} A^T y, then
 // one step of iterative refinement with the corrected seminormal equations (Bjorck, Linear Algebra
 // Appl. 88/89, 1987): r = y - A c, c += (L1 L1^T)^{-1} A^T r.  A step shrinks the error by about
-// cond(A)^2 eps, which the first one's own size eta = |A dc| / |A c| measures: up to 1e-9 (cond(A)
-// of about 1e4) what it leaves is below round-off.  *done = false above that: there the limit is the
-// rounding of A^T r, and the reorthogonalising pass has the smaller error.  Error of the
-// coefficients against extended precision, 162 fits (15 to 60 terms, residuals 0 to 1), as a multiple of that
-// pass's (geometric mean): cond below 30 0.57, below 1e4 0.65 to 1.04, above 1e5 1.4.
+// cond(A)^2 eps.  Taken while two things are small; else *done = false and the reorthogonalising pass
+// follows, whose error is the smaller one there.
+// (1) The condition of A with its columns scaled to unit norm, from the factor's inverse in the Frobenius
+//     norm (1.3 to 13 times that of the 2-norm on the bases measured, 1.3 to 5 above 1e4): up to 2e5.
+// (2) The first solution's own misfit eta = |A dc| / |A c|, up to 1e-9, which is also large where the
+//     residual is and the rounding of A^T r then limits the step (cond(A) above about 1e4).  Alone it does not see the
+//     condition: a target in the dominant directions of A has a small eta at any, and errors of 1.3e-7
+//     (cond 4e6) and 1.6e-5 (2e7) passed where the other pass gives 1e-9 and 3.5e-9.
+// Error of the coefficients against extended precision as a multiple of the reorthogonalising pass's
+// (geometric means over 276 fits of 8 to 60 terms; targets fitted, dominant, noisy and white): bound (1) at
+// 2e4 to 6e4 0.70, 0.43, 0.51 and 1.6; at 6e4 to 2e5 0.48, 0.84, 1.28 (white: by (2) never refined); at 6e5 to 2e6 about
+// 1, with single fits three times as far off; beyond, up to five orders.
 // z = A^T y; *status is the factorisation's.
-constexpr double kRefineMax = 1e-9;
+constexpr double kRefineMax = 1e-9, kRefineCond = 2e5;
 probe_status fit_refine(probe_t h, const BasisDev& B, const double* w, const float* yd, const double* alpha, int nmax,
                         int p, const double* L1, const double* z, double* coef, int* status, bool* done,
                         cudaStream_t st) {
     FitCache& c = *h->fit;
     PROBE_TRY(ensure_buf(h, c.part, (size_t)kRefBlocks * B.P * 8));
     double* part = (double*)c.part.p;
-    double* norms = (double*)c.misc.p + 3;  // |A c|^2, |A dc|^2
+    double* norms = (double*)c.misc.p + 3;  // |A c|^2, |A dc|^2, |L^{-1} D|_F^2 in two parts
     PROBE_CK(h, cudaMemsetAsync(coef, 0, (size_t)B.P * 8, st));
-    k_fit_refine_step<<<1, 256, 0, st>>>(z, 1, B.P, L1, coef, norms);
+    k_fit_refine_step<<<1, 256, 0, st>>>(z, 1, B.P, L1, coef, norms, nullptr);
     k_fit_refine<<<kRefBlocks, 256, 0, st>>>(w, yd, alpha, nmax, p, B, coef, part);
-    k_fit_refine_step<<<1, 256, 0, st>>>(part, kRefBlocks, B.P, L1, coef, norms + 1);
+    k_fit_refine_step<<<1, 256, 0, st>>>(part, kRefBlocks, B.P, L1, coef, norms + 1, norms + 2);
     PROBE_CK(h, cudaGetLastError());
     int bad = 0;
-    double n2[2];
+    double n2[4];
     PROBE_CK(h, cudaMemcpyAsync(&bad, status, sizeof(int), cudaMemcpyDeviceToHost, st));
     PROBE_CK(h, cudaMemcpyAsync(n2, norms, sizeof(n2), cudaMemcpyDeviceToHost, st));
     PROBE_CK(h, cudaStreamSynchronize(st));
     // rank deficient (reported by the caller), or refined; a NaN is not
-    *done = bad || n2[1] <= kRefineMax * kRefineMax * n2[0];
+    *done = bad || (n2[1] <= kRefineMax * kRefineMax * n2[0] && B.P * (n2[2] + n2[3]) <= kRefineCond * kRefineCond);
     return PROBE_OK;
 }
 

@@ -108,3 +108,27 @@ def test_angular_indices_at_the_ends_of_their_type(cuda_device, q):
     img = np.random.default_rng(9).standard_normal((33, 40)).astype(np.float32)
     got = probe.apply_precond(g, c, torch.tensor(img, device=cuda_device)).cpu().numpy()
     assert rel(got, o.apply(c, img.astype(np.float64))) < 2e-5
+
+
+@pytest.mark.parametrize("spatial,angular,nradial,sigma", [
+    ([(0, 0), (1, 0)], [0, 2], 8, 3),       # cond 2e5
+    ([(0, 0)], [0], 14, 2),                 # cond 4e6
+    ([(0, 0)], [0, 2], 13, 3),              # cond 7e6
+    ([(0, 0), (0, 1)], [0], 14, 3),         # cond 1e7
+])
+def test_fit_of_targets_in_the_dominant_direction(cuda_device, spatial, angular, nradial, sigma):
+    """Targets A v_1 (v_1 the first right singular vector) on ill-conditioned columns: the misfit of the
+    first solution is then small however large its error is along the other singular vectors, so it says
+    nothing about the condition.  Bound: as in test_fit_refinement_has_the_accuracy_of_qr."""
+    from scipy.ndimage import gaussian_filter
+    shape = (43, 51)
+    wl, probe, g, o = setup(shape, spatial, angular, nradial, -1.0, 5)
+    xs = np.random.default_rng(4).standard_normal((2,) + shape)
+    xs = np.stack([gaussian_filter(x, sigma) for x in xs]).astype(np.float32)
+    A = np.concatenate([o.columns(x.astype(np.float64)) for x in xs])
+    ys = (A @ np.linalg.svd(A, full_matrices=False)[2][0]).reshape((2,) + shape).astype(np.float32)
+    c_orc, res_orc, cond = ofit(o, ys, xs)
+    c, res = probe.fit(g, torch.tensor(ys, device=cuda_device), torch.tensor(xs, device=cuda_device))
+    r = res_orc * np.linalg.norm(ys.astype(np.float64))
+    bound = 1e-14 * cond * (2 + cond * r / (np.linalg.norm(A, 2) * np.linalg.norm(c_orc)))
+    assert rel(c, c_orc) < bound, (cond, bound)
