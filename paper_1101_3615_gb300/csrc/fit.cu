@@ -1066,7 +1066,9 @@ probe_status fit_gram(probe_t h, const BasisDev& B, const double* w, const float
         if (!L1 && B.nspatial > 1 && sm <= kGramSmemMax) {
             const int nout = gram_plan(B).nout;
             PROBE_TRY(ensure_buf(h, c.part, (size_t)kGramBlocks * nout * 8));
-            PROBE_CK(h, cudaFuncSetAttribute(k_fit_gram_s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+            // the most that any basis takes, not this one's: another thread's call may set it before the launch
+            PROBE_CK(h, cudaFuncSetAttribute(k_fit_gram_s, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kGramSmemMax));
             k_fit_gram_s<<<kGramBlocks, 256, sm, st>>>(w, yd, alpha, nmax, p, B, (double*)c.part.p);
             k_fit_out_to_C<<<grid_of(32ll * nout), 256, 0, st>>>((const double*)c.part.p, kGramBlocks, B, C);
             PROBE_CK(h, cudaGetLastError());

@@ -132,3 +132,31 @@ def test_fit_of_targets_in_the_dominant_direction(cuda_device, spatial, angular,
     r = res_orc * np.linalg.norm(ys.astype(np.float64))
     bound = 1e-14 * cond * (2 + cond * r / (np.linalg.norm(A, 2) * np.linalg.norm(c_orc)))
     assert rel(c, c_orc) < bound, (cond, bound)
+
+
+def test_fits_from_two_threads(cuda_device):
+    """Handles of their own, streams of their own, staged factors of different size: the same results as alone."""
+    import threading
+    todo, errors = [], []
+    for spatial, angular, nradial in (([(0, 0), (0, 1)], [0, 2, -2, 4, -4, 6, -6, 8], 3), ([(0, 0), (0, 1)], [0], 2)):
+        wl, probe, g, o = setup((24, 27), spatial, angular, nradial, -1.0, 2)
+        xs = np.random.default_rng(4).standard_normal((2, 24, 27)).astype(np.float32)
+        ys = np.random.default_rng(5).standard_normal((2, 24, 27)).astype(np.float32)
+        xs, ys = torch.tensor(xs, device=cuda_device), torch.tensor(ys, device=cuda_device)
+        todo.append((probe, g, ys, xs, probe.fit(g, ys, xs)[0]))
+    torch.cuda.synchronize()
+
+    def work(probe, g, ys, xs, ref):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(200):
+                    assert np.array_equal(probe.fit(g, ys, xs)[0], ref)
+        except Exception as e:  # reported by the test's own thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=t) for t in todo]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
