@@ -117,9 +117,8 @@ typedef enum {
     PROBE_OPT_TILE_Z = 6,        /* 2D tile height override (16 or 32); 0 = default */
     PROBE_OPT_PIPELINE = 7,      /* 2D: 0 = one tile per CTA; 2 or 3 = persistent warp-specialised
                                     CTAs with a 2- or 3-stage TMA ring (tiles 64 x 16R, see
-                                    PROBE_OPT_PIPE_ROWS), for the forward and the adjoint.  The
-                                    pipelined variants give the same bits, and those of one tile
-                                    per CTA up to rounding on all-interior tiles.  3D: 0 = one-barrier-per-plane
+                                    PROBE_OPT_PIPE_ROWS), for the forward and the adjoint.  Every
+                                    variant gives the same bits.  3D: 0 = one-barrier-per-plane
                                     kernels; 2 = pipelined kernels whose ring is refilled by a
                                     producer warp; 3 = pipelined kernels whose ring slot is refilled
                                     by the last compute warp done with it (no producer warp); by

@@ -132,8 +132,8 @@ __device__ __forceinline__ void cluster_sync_all() {
 // Rounding-explicit pieces of the explicit time update u^{n+1} = G (2 u^n - a- u^{n-1} + rhs)
 // (Sec. 2 scheme with the sponge).  Every product and sum is one IEEE operation written
 // out, so the compiler cannot fuse them differently in different kernel instantiations:
-// the 2D variants give the same bits (the pipelined kernels' packed all-interior path excepted, where
-// the compiler fuses a product and a sum).
+// all 2D variants (one tile per CTA, pipelined, cluster-resident, single- or multi-model) give the same
+// bits.
 __device__ __forceinline__ float leapfrog(float G, float c, float am, float prev, float rhs) {
     return __fmul_rn(G, __fadd_rn(__fmaf_rn(-am, prev, __fadd_rn(c, c)), rhs));
 }
@@ -207,9 +207,15 @@ __device__ __forceinline__ P4 p4fma(const P4& x, const P4& y, const P4& z) {
 __device__ __forceinline__ P4 p4neg(const P4& x) {
     return {make_float2(-x.a.x, -x.a.y), make_float2(-x.b.x, -x.b.y)};
 }
+// x + y with one rounding where x is a product.  ptxas contracts a packed product and a packed sum into
+// one fused multiply-add even where both are written with .rn; a fused multiply-add by a factor it cannot
+// know (one = 1, a kernel parameter) keeps the product's own rounding, at the cost of the sum.
+__device__ __forceinline__ P4 p4add_one(const P4& x, const P4& y, float one) {
+    return p4fma(x, p4(one, one, one, one), y);
+}
 // leapfrog() of an interior cell (G = a- = 1): (2c - prev) + rhs; the factor G = 1 is exact.
-__device__ __forceinline__ P4 p4leap1(const P4& c, const P4& prev, const P4& rhs) {
-    return p4add(p4sub(p4add(c, c), prev), rhs);
+__device__ __forceinline__ P4 p4leap1(const P4& c, const P4& prev, const P4& rhs, float one) {
+    return p4add_one(rhs, p4sub(p4add(c, c), prev), one);
 }
 
 // Bring the line holding p into L2 (a hint: no registers held, nothing returned).

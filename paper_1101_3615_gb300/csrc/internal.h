@@ -104,6 +104,7 @@ struct StepParams2D {
     int n;    // time index of the step (forward: u^n -> u^{n+1}; adjoint: computes mu^n)
     int two;  // time-blocked forward kernel: 1 = advance n -> n + 2, 0 = one step
     int nt;
+    float one;  // 1, unknown to the compiler (pipelined forward kernels; set with the sweep)
     int* err; // device error word
     ModelStep2D m[kMaxModels];
 };

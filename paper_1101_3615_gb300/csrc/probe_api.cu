@@ -599,6 +599,7 @@ probe_status prepare_sweep(Sweep& sw, probe_t h0, cudaStream_t st) {
     memset(&sw.pa, 0, sizeof(sw.pa));
     sw.pa.nmodels = sw.p.nmodels;
     sw.pa.nt = sw.p.nt;
+    sw.p.one = sw.pa.one = 1.f;
     sw.pa.err = sw.p.err;
     sw.st = st;
     sw.nt = h0->nt;

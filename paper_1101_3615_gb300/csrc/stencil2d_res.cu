@@ -36,13 +36,6 @@ namespace {
 constexpr int kResThreads = 512;
 constexpr int kResPadMax = 64;  // sponge table of at most 17 KB
 
-// x + y with one rounding.  ptxas contracts a packed product and a packed sum into one fused
-// multiply-add even where both are written with .rn; a fused multiply-add by a factor it cannot know
-// (one = 1, a kernel parameter) keeps the product's own rounding, at the cost of the sum.
-__device__ __forceinline__ P4 p4add_one(const P4& x, const P4& y, float one) {
-    return p4fma(x, p4(one, one, one, one), y);
-}
-
 // 16 bytes from global to shared memory without passing through registers
 __device__ __forceinline__ void cp_async16(float* dst, const float* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");

@@ -51,10 +51,6 @@ __device__ __forceinline__ float q_sponge_e(const ModelStep3D& M, int z, int y, 
     return __fmaf_rn(M.cz, (float)(rz * rz), __fmaf_rn(M.cy, (float)(ry * ry), __fmul_rn(M.cx, (float)(rx * rx))));
 }
 
-// x + y with one rounding, safe from contraction with the product that formed x (one = 1, unknown to
-// the compiler; ptxas fuses a packed product and a packed sum otherwise).
-__device__ __forceinline__ P4 q_add(const P4& x, const P4& y, float one) { return p4fma(x, p4(one, one, one, one), y); }
-
 template <int MODE, int NI>
 __global__ void __launch_bounds__(kThreads + 32, 2) k_step3d_q(const __grid_constant__ StepParams3D p) {
     using O = QOps<MODE, NI>;
@@ -276,11 +272,11 @@ __global__ void __launch_bounds__(kThreads + 32, 2) k_step3d_q(const __grid_cons
                         if (x + j >= M.Nx) g[j] = 0.f;
                     }
                     o = f4(p4mul(p4(g[0], g[1], g[2], g[3]),
-                                 q_add(Fo, p4fma(p4neg(p4(a[0], a[1], a[2], a[3])), prev, c2), one)));
+                                 p4add_one(Fo, p4fma(p4neg(p4(a[0], a[1], a[2], a[3])), prev, c2), one)));
                 } else if (tile_in) {
-                    o = f4(q_add(Fo, p4sub(c2, prev), one));
+                    o = f4(p4add_one(Fo, p4sub(c2, prev), one));
                 } else {
-                    o = f4(p4mul(p4(Gc), q_add(Fo, p4fma(p4neg(p4(Ac)), prev, c2), one)));
+                    o = f4(p4mul(p4(Gc), p4add_one(Fo, p4fma(p4neg(p4(Ac)), prev, c2), one)));
                 }
                 st4(outp, o);
                 if (INC && auxp) {
