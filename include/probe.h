@@ -170,9 +170,10 @@ typedef enum {
 /* Counters and timings of the last apply call (probe_get_stats). */
 typedef struct {
     double ms_forward;           /* forward (incident + Born) sweeps, CUDA events */
-    double ms_recompute;         /* checkpoint recompute sweeps */
+    double ms_recompute;         /* checkpoint recompute sweeps (cluster-resident kernels, whose recompute
+                                    runs beside the adjoint: what the adjoint waits for) */
     double ms_adjoint;           /* adjoint + imaging sweeps */
-    double ms_total;             /* whole call on the device */
+    double ms_total;             /* the sum of these */
     long long launches_forward;  /* kernel launches in each sweep kind */
     long long launches_recompute;
     long long launches_adjoint;
@@ -233,9 +234,12 @@ probe_status probe_apply_H(probe_t h, const float* dm, float* Hdm, int nb,
                            probe_stream_t stream);
 
 /* probe_apply_H on several models (of possibly different grid sizes) at once:
- * the sweeps of all models advance in the same kernel launches.  All models
+ * the sweeps of all models advance in the same kernel launches, or, where every
+ * grid fits a cluster's shared memory and that is estimated faster, model after
+ * model on the cluster-resident kernels.  All models
  * must share nt, dt and the checkpoint stride.  dm[k], Hdm[k] are the arrays
- * of model k with nb[k] trials each.  nmodels <= 4. */
+ * of model k with nb[k] trials each.  nmodels <= 4.  The statistics are kept on
+ * models[0] and cover the whole group. */
 probe_status probe_apply_H_group(const probe_t* models, int nmodels,
                                  const float* const* dm, float* const* Hdm,
                                  const int* nb, probe_stream_t stream);

@@ -1002,7 +1002,8 @@ probe_status run_forward_res(Sweep& sw, Job& jb, const ResSet& rs, FwdKind kind,
     return PROBE_OK;
 }
 
-probe_status run_adjoint_res(Sweep& sw, Job& jb, const ResSet& rs) {
+// Timing events go to ht, from *ev on (a group's models, one after the other, share the first one's).
+probe_status run_adjoint_res(Sweep& sw, Job& jb, const ResSet& rs, probe_t ht, int* ev) {
     probe_t h = jb.h;
     Workspace& w = h->ws;
     cudaStream_t st = sw.st;
@@ -1026,11 +1027,10 @@ probe_status run_adjoint_res(Sweep& sw, Job& jb, const ResSet& rs) {
     cudaStream_t su = h->ostream;
     CK(h, cudaEventRecord(h->ov_inc[0], st));
     CK(h, cudaStreamWaitEvent(su, h->ov_inc[0], 0));
-    int ev = 2;
     for (int k = h->nck - 1, i = 0; k >= 0; --k) {
         const int k0 = k * h->K, k1 = std::min(k0 + h->K, h->nt - 1), set = i & 1;
         if (k0 >= k1) continue;
-        record(h, ev++, st);
+        record(ht, (*ev)++, st);
         if (i >= 2) CK(h, cudaStreamWaitEvent(su, h->ov_born[set], 0));
         cudaError_t e = cudaSuccess;
         if (h->snap == PROBE_SNAP_FP32) {
@@ -1060,7 +1060,7 @@ probe_status run_adjoint_res(Sweep& sw, Job& jb, const ResSet& rs) {
         sw.launches_rec++;
         CK(h, cudaEventRecord(h->ov_inc[set], su));
         CK(h, cudaStreamWaitEvent(st, h->ov_inc[set], 0));
-        record(h, ev++, st);
+        record(ht, (*ev)++, st);
         pa.n0 = k1;
         pa.nsteps = k1 - k0;
         pa.slot0 = set * h->K + (k1 - k0 - 1);  // level n uses Dtt u^{n-1}
@@ -1072,7 +1072,7 @@ probe_status run_adjoint_res(Sweep& sw, Job& jb, const ResSet& rs) {
         sw.launches_adj++;
         ++i;
     }
-    record(h, ev++, st);
+    record(ht, (*ev)++, st);
     return PROBE_OK;
 }
 
@@ -2123,6 +2123,44 @@ probe_status autotune_2d(probe_t h, const std::vector<long long>& key, std::vect
     return PROBE_OK;
 }
 
+// Executed cell updates and algorithmic bytes of one job's sweeps (a shot wave of one model), added to
+// the statistics.  res: on the cluster-resident kernels; tb2: 2D with two levels per launch.
+void add_counts(probe_stats& s, const Job& jb, FwdKind kind, bool need_ckpt, bool res, bool tb2) {
+    probe_t h = jb.h;
+    const Workspace& w = h->ws;
+    const int nb = jb.nb;
+    const double updates = (double)h->Nz * h->Ny * h->Nx * (h->nt - 1);  // of one field
+    s.cell_updates_forward += updates * jb.W * (kind == FWD_BORN ? 1 + nb : 1);
+    // algorithmic bytes: incident 16 B (u^n, u^{n-1}, s, write), Born +16 B per trial
+    // (du^n, du^{n-1}, dm, write); +4 B Dtt write in the recompute.  The 3D one-field kernels
+    // (no cluster fusion) also write Dtt u^n (4 B) and read it and s once per trial (8 B).
+    const bool hist = w.history != 0;
+    const bool split3 = h->ndim == 3 && kind == FWD_BORN && !((h->opt_cluster3d & 1) && nb + 1 <= 8);
+    // two levels per launch: per cell and level (10 + 10 nb) bytes for the Born forward (u^n,
+    // u^{n-1}, s, two writes, per trial likewise, every other level) and 14 bytes for the
+    // recompute (with its two Dtt writes)
+    if (res)  // the fields stay on chip: Dtt u^n written once and read once per trial
+        s.bytes_forward += kind == FWD_BORN ? updates * jb.W * (4.0 + 4.0 * nb) : 0.0;
+    else if (tb2 && kind == FWD_BORN)
+        s.bytes_forward += updates * jb.W * (10.0 + 10.0 * nb + (hist ? 4.0 : 0.0));
+    else
+        s.bytes_forward += updates * jb.W * (16.0 + (kind == FWD_BORN ? 16.0 * nb : 0.0) + (hist ? 4.0 : 0.0) +
+                                             (split3 ? 4.0 + 8.0 * nb : 0.0));
+    if (!need_ckpt) return;
+    if (!hist) {
+        s.cell_updates_recompute += updates * jb.W;
+        s.bytes_recompute += updates * jb.W * (res ? 4.0 : tb2 ? 14.0 : 20.0);
+    }
+    s.cell_updates_adjoint += updates * jb.W * nb;
+    // adjoint: per (shot, trial) mu^{n+1}, mu^{n+2}, write mu^n = 12 B; per shot Dtt 4 B;
+    // s 4 B and image traffic per (group, trial) amortised over the group
+    // (3D one-field adjoint with Kahan: 8 B segment-image read-modify-write per step, the
+    //  Kahan fold of 20 B per cell once per segment)
+    const double img_b = w.seg ? 8.0 + 20.0 / h->K : (h->kahan ? 16.0 : 8.0);
+    s.bytes_adjoint += res ? updates * 4.0 * jb.W * nb
+                           : updates * (12.0 * jb.W * nb + 4.0 * jb.W + (double)jb.groups * (4.0 + img_b * nb));
+}
+
 // Run one operator on one model.  dm: device [nb][n]; data_user: device [nb][ns][nt][nr] (F / F*)
 // or [ns][nt][nr] (nonlinear / gradient); img_out: device [nb][n].
 probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in, float* data_out,
@@ -2253,7 +2291,8 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
                 record(h, 0, ss);
                 TRY(rs.use ? run_forward_res(sw2, sw2.jobs[0], rs, kind, need_ckpt) : run_forward(sw2, kind, need_ckpt));
                 record(h, 1, ss);
-                if (need_ckpt) TRY(rs.use ? run_adjoint_res(sw2, sw2.jobs[0], rs) : run_adjoint(sw2));
+                int ev = 2;
+                if (need_ckpt) TRY(rs.use ? run_adjoint_res(sw2, sw2.jobs[0], rs, h, &ev) : run_adjoint(sw2));
                 cnt[0] = sw2.launches_fwd;
                 cnt[1] = sw2.launches_rec;
                 cnt[2] = sw2.launches_adj;
@@ -2266,43 +2305,8 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
             sw.launches_other = cnt[3];
             finish_stats(h, sw, nwaves);
         }
-        const double cells = (double)h->Nz * h->Ny * h->Nx;
-        const double steps = h->nt - 1;
-        const int nfields = (kind == FWD_BORN) ? 1 + nbw : 1;
-        h->stats.cell_updates_forward += cells * steps * Wv * nfields;
-        // algorithmic bytes: incident 16 B (u^n, u^{n-1}, s, write), Born +16 B per trial
-        // (du^n, du^{n-1}, dm, write); +4 B Dtt write in the recompute.  The 3D one-field kernels
-        // (no cluster fusion) also write Dtt u^n (4 B) and read it and s once per trial (8 B).
-        const bool hist = w.history != 0;
-        const bool split3 = h->ndim == 3 && kind == FWD_BORN && !((h->opt_cluster3d & 1) && nbw + 1 <= 8);
-        // 2D with two levels per launch: per cell and level (10 + 10 nb) bytes for the Born
-        // forward (u^n, u^{n-1}, s, two writes, per trial likewise, every other level) and 14 bytes
-        // for the recompute (with its two Dtt writes)
-        const bool tb2 = h->ndim == 2 && h->opt_tblock == 2 && h->tile_z == kPipeTZ && w.u4;
-        if (rs.use)  // the fields stay on chip: Dtt u^n written once and read once per trial
-            h->stats.bytes_forward += kind == FWD_BORN ? cells * steps * Wv * (4.0 + 4.0 * nbw) : 0.0;
-        else if (tb2 && kind == FWD_BORN)
-            h->stats.bytes_forward += cells * steps * Wv * (10.0 + 10.0 * nbw + (hist ? 4.0 : 0.0));
-        else
-            h->stats.bytes_forward += cells * steps * Wv *
-                                      (16.0 + (kind == FWD_BORN ? 16.0 * nbw : 0.0) + (hist ? 4.0 : 0.0) +
-                                       (split3 ? 4.0 + 8.0 * nbw : 0.0));
-        if (need_ckpt) {
-            if (!hist) {
-                h->stats.cell_updates_recompute += cells * steps * Wv;
-                h->stats.bytes_recompute += cells * steps * Wv * (rs.use ? 4.0 : tb2 ? 14.0 : 20.0);
-            }
-            h->stats.cell_updates_adjoint += cells * steps * Wv * nbw;
-            // adjoint: per (shot, trial) mu^{n+1}, mu^{n+2}, write mu^n = 12 B; per shot Dtt 4 B;
-            // s 4 B and image traffic per (group, trial) amortised over the group
-            // (3D one-field adjoint with Kahan: 8 B segment-image read-modify-write per step, the
-            //  Kahan fold of 20 B per cell once per segment)
-            const bool seg3 = w.seg != nullptr;
-            const double img_b = seg3 ? 8.0 + 20.0 / h->K : (h->kahan ? 16.0 : 8.0);
-            h->stats.bytes_adjoint += rs.use ? cells * steps * 4.0 * Wv * nbw
-                                             : cells * steps * (12.0 * Wv * nbw + 4.0 * Wv +
-                                                                (double)jb.groups * (4.0 + img_b * nbw));
-        }
+        add_counts(h->stats, jb, kind, need_ckpt, rs.use,
+                   h->ndim == 2 && h->opt_tblock == 2 && h->tile_z == kPipeTZ && w.u4);
     }
     h->ev_base = 0;
     if (need_ckpt && img_out) {
@@ -2586,7 +2590,8 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
     h0->stats.pipeline_adjoint = res ? 1 : (piped ? h0->pipe_adj : 0);
     h0->stats.pipeline_rows = piped ? h0->ws_rows : 0;
     h0->stats.pipeline_rows_adjoint = piped ? h0->ws_rows_adj : 0;
-    if (h0->opt_timing) TRY(ensure_events(h0, 3 + 2 * h0->nck + 2));
+    h0->stats.time_block = res ? h0->K : h0->tile_z == kPipeTZ && h0->ws.u4 ? h0->opt_tblock : 1;
+    if (h0->opt_timing) TRY(ensure_events(h0, 2 + (res ? nmodels : 1) * (2 * h0->nck + 3)));
     // the whole group's sweeps as one graph (cached on h0 by handles, workspaces and variants)
     std::vector<long long> gkey = key;
     for (const Job& jb : sw.jobs) {
@@ -2609,7 +2614,8 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
             record(h0, 0, ss);
             for (int k = 0; k < nmodels; ++k) TRY(run_forward_res(sw2, sw2.jobs[k], rss[k], FWD_BORN, true));
             record(h0, 1, ss);
-            for (int k = 0; k < nmodels; ++k) TRY(run_adjoint_res(sw2, sw2.jobs[k], rss[k]));
+            int ev = 2;
+            for (int k = 0; k < nmodels; ++k) TRY(run_adjoint_res(sw2, sw2.jobs[k], rss[k], h0, &ev));
         } else {
             TRY(prepare_sweep(sw2, h0, ss));
             record(h0, 0, ss);
@@ -2635,28 +2641,23 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
         cudaError_t e = launch_extract_images(w.img, w.comp, groups_k, (long long)nb[k] * h->F, nb[k], h->F, outs[k],
                                               h->nz, 1, h->nx, h->pad, 1, h->P, h->kahan != 0, false, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "image extraction");
-        const double cells = (double)h->Nz * h->Nx, steps = h->nt - 1;
-        h0->stats.cell_updates_forward += cells * steps * h->ns * (1 + nb[k]);
-        h0->stats.cell_updates_recompute += cells * steps * h->ns;
-        h0->stats.cell_updates_adjoint += cells * steps * h->ns * nb[k];
-        // algorithmic bytes, as for probe_apply_H
-        h0->stats.bytes_forward += cells * steps * h->ns * (16.0 + 16.0 * nb[k]);
-        h0->stats.bytes_recompute += cells * steps * h->ns * 20.0;
-        h0->stats.bytes_adjoint += cells * steps * (12.0 * h->ns * nb[k] + 4.0 * h->ns +
-                                                    (double)sw.jobs[k].groups * (4.0 + (h->kahan ? 16.0 : 8.0) * nb[k]));
+        add_counts(h0->stats, sw.jobs[k], FWD_BORN, true, res,
+                   h0->opt_tblock == 2 && h0->tile_z == kPipeTZ && h0->ws.u4);
         TRY(finish_call(h, st, any_host, outs[k], (long long)nb[k] * h->nmodel));
     }
     if (h0->opt_timing) {
         CK(h0, cudaStreamSynchronize(st));
         h0->stats.ms_forward = elapsed(h0, 0, 1);
-        int ev = 2;
-        for (int kk = h0->nck - 1; kk >= 0; --kk) {
-            const int k0 = kk * h0->K, k1 = std::min(k0 + h0->K, h0->nt - 1);
-            if (k0 >= k1) continue;
-            h0->stats.ms_recompute += elapsed(h0, ev, ev + 1);
-            h0->stats.ms_adjoint += elapsed(h0, ev + 1, ev + 2);
-            ev += 2;
-        }
+        if (h0->opt_timing == 1 && h0->ws.history) h0->stats.ms_adjoint = elapsed(h0, 3, 4);
+        const int sweeps = h0->opt_timing != 1 || h0->ws.history ? 0 : res ? nmodels : 1;  // resident: model after model
+        for (int k = 0, ev = 2; k < sweeps; ++k, ++ev)
+            for (int kk = h0->nck - 1; kk >= 0; --kk) {
+                const int k0 = kk * h0->K, k1 = std::min(k0 + h0->K, h0->nt - 1);
+                if (k0 >= k1) continue;
+                h0->stats.ms_recompute += elapsed(h0, ev, ev + 1);
+                h0->stats.ms_adjoint += elapsed(h0, ev + 1, ev + 2);
+                ev += 2;
+            }
         h0->stats.ms_total = h0->stats.ms_forward + h0->stats.ms_recompute + h0->stats.ms_adjoint;
     }
     for (int k = 0; k < nmodels; ++k) {

@@ -1,0 +1,75 @@
+"""Counters and times of probe_get_stats on the cluster-resident 2D path and on groups.
+
+Counts: a group's are the sum of its models' own.  Times: a group's cover all of its models, and a group
+leaves the times of an earlier call on another of its handles alone (factors of two and more apart, so
+that timer noise does not matter).
+"""
+import numpy as np
+import pytest
+
+from workloads import mini_config
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def probe_of(wl, **kw):
+    from paper_1101_3615_gb300 import Probe
+    return Probe(wl.m0, wl.h, wl.dt, wl.nt, wl.pad, wl.src, wl.rec, wl.wavelet, **kw)
+
+
+def workload(shape, nt, ns, nb, cfg=3):
+    wl = mini_config(cfg, shape=shape, nt=nt, ns=ns, pad=6, p=1)
+    rng = np.random.default_rng(2)
+    wl.trials = (rng.standard_normal((nb,) + tuple(shape)) * 0.05 * wl.m0.mean()).astype(np.float32)
+    return wl
+
+
+COUNTS = ["cell_updates_forward", "cell_updates_recompute", "cell_updates_adjoint",
+          "bytes_forward", "bytes_recompute", "bytes_adjoint"]
+
+
+@pytest.mark.parametrize("resident", [True, False])
+def test_group_counts_are_the_sum_of_its_models(cuda_device, resident):
+    from paper_1101_3615_gb300 import apply_H_group
+    wls = [workload((61, 45), 90, 3, 1), workload((40, 70), 90, 2, 3)]
+    probes = [probe_of(w) for w in wls]
+    if not resident:
+        for p in probes:
+            p.set_option("pipeline", 2)
+            p.set_option("shot_group", 2)
+    dms = [torch.tensor(w.trials, device=cuda_device) for w in wls]
+    solo = []
+    for p, d in zip(probes, dms):
+        p.apply_H(d)
+        solo.append(p.stats())
+    apply_H_group(probes, dms)
+    s = probes[0].stats()
+    assert (s["pipeline_forward"] == 1) == resident
+    for k in COUNTS:
+        assert s[k] == pytest.approx(sum(x[k] for x in solo), rel=1e-12), k
+
+
+def test_resident_group_times_cover_every_model(cuda_device):
+    from paper_1101_3615_gb300 import apply_H_group
+    small, large = workload((30, 30), 300, 1, 1), workload((150, 160), 300, 8, 24)
+    ps, pl = probe_of(small), probe_of(large)
+    ds, dl = (torch.tensor(w.trials, device=cuda_device) for w in (small, large))
+    for p in (ps, pl):
+        p.set_option("timing", 1)
+    one = dl[:1].contiguous()
+    solo, single = [], []
+    for _ in range(3):
+        pl.apply_H(dl)
+        solo.append(pl.stats())
+        pl.apply_H(one)
+        single.append(pl.stats()["ms_adjoint"])
+        apply_H_group([ps, pl], [ds, dl])
+    pl.apply_H(one)                       # its times are formed when they are read, after the group call
+    apply_H_group([ps, pl], [ds, dl])
+    late = pl.stats()["ms_adjoint"]
+    g = ps.stats()
+    for k in ("ms_forward", "ms_adjoint", "ms_total"):
+        assert g[k] > 0.7 * min(s[k] for s in solo), k
+    assert min(s["ms_adjoint"] for s in solo) > 2.5 * max(single)
+    assert late < 1.5 * max(single)
