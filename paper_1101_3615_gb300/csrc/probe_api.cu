@@ -2153,12 +2153,22 @@ void add_counts(probe_stats& s, const Job& jb, FwdKind kind, bool need_ckpt, boo
     }
     s.cell_updates_adjoint += updates * jb.W * nb;
     // adjoint: per (shot, trial) mu^{n+1}, mu^{n+2}, write mu^n = 12 B; per shot Dtt 4 B;
-    // s 4 B and image traffic per (group, trial) amortised over the group
-    // (3D one-field adjoint with Kahan: 8 B segment-image read-modify-write per step, the
-    //  Kahan fold of 20 B per cell once per segment)
-    const double img_b = w.seg ? 8.0 + 20.0 / h->K : (h->kahan ? 16.0 : 8.0);
+    // s 4 B and image traffic per (group, trial) amortised over the group: 8 B (with Kahan 16 B) per update.
+    // 3D segment images: 8 B per update but for a segment's first, which reads nothing, and the fold of
+    // 20 B once per segment.  The register-queue kernels update an image every third step of a segment.
+    double img_b = (h->kahan ? 16.0 : 8.0) * (h->nt - 1);  // of one cell over the sweep
+    if (h->ndim == 3) {
+        const bool queue = h->pipe_adj == 4 && adj3d_ws(h) && (h->nband == 0 || w.inj);
+        const bool plain = w.seg || !h->kahan;
+        if (plain) img_b = 0.0;
+        for (int k0 = 0; plain && k0 < h->nt - 1; k0 += h->K) {
+            const int T = std::min(h->K, h->nt - 1 - k0);
+            img_b += 8.0 * (queue ? (T + 2) / 3 : T) + (w.seg ? 20.0 - 4.0 : 0.0);
+        }
+    }
     s.bytes_adjoint += res ? updates * 4.0 * jb.W * nb
-                           : updates * (12.0 * jb.W * nb + 4.0 * jb.W + (double)jb.groups * (4.0 + img_b * nb));
+                           : updates * (12.0 * jb.W * nb + 4.0 * jb.W +
+                                        (double)jb.groups * (4.0 + img_b / (h->nt - 1) * nb));
 }
 
 // Run one operator on one model.  dm: device [nb][n]; data_user: device [nb][ns][nt][nr] (F / F*)

@@ -1,9 +1,12 @@
-"""Counters and times of probe_get_stats on the cluster-resident 2D path and on groups.
+"""Counters and times of probe_get_stats on the cluster-resident 2D path, on groups and in 3D.
 
-Counts: a group's are the sum of its models' own.  Times: a group's cover all of its models, and a group
-leaves the times of an earlier call on another of its handles alone (factors of two and more apart, so
-that timer noise does not matter).
+Counts: a group's are the sum of its models' own; the bytes of a 3D adjoint are its model written out
+segment by segment.  Times: a group's cover all of its models, and a group leaves the times of an
+earlier call on another of its handles alone (factors of two and more apart, so that timer noise does
+not matter).
 """
+import math
+
 import numpy as np
 import pytest
 
@@ -73,3 +76,27 @@ def test_resident_group_times_cover_every_model(cuda_device):
         assert g[k] > 0.7 * min(s[k] for s in solo), k
     assert min(s["ms_adjoint"] for s in solo) > 2.5 * max(single)
     assert late < 1.5 * max(single)
+
+
+@pytest.mark.parametrize("nt,K", [(40, 0), (32, 5), (20, 1)])
+@pytest.mark.parametrize("kahan", [True, False])
+@pytest.mark.parametrize("pipeline", [None, 2])
+def test_adjoint_3d_bytes(cuda_device, nt, K, kahan, pipeline):
+    wl = workload((20, 18, 22), nt, 1, 3, cfg=5)
+    wl.src = np.array([[2, 5, 6], [3, 12, 15]], np.int32)
+    p = probe_of(wl, ckpt_stride=K, kahan=kahan)
+    if pipeline:
+        p.set_option("pipeline", pipeline)
+    p.apply_H(torch.tensor(wl.trials, device=cuda_device))
+    s = p.stats()
+    assert s["pipeline_adjoint"] == (pipeline or 4)
+    stride = s["ckpt_stride"]
+    per_cell = 0.0                        # of one (shot, trial); Dtt and s of a shot are shared by its trials
+    for k0 in range(0, nt - 1, stride):
+        T = min(stride, nt - 1 - k0)
+        touches = math.ceil(T / 3) if not pipeline else T      # image updates of the segment
+        per_cell += 12.0 * T + (4.0 + 4.0) * T / 3 + 8.0 * touches
+        if kahan:
+            per_cell += 20.0 - 4.0        # the fold; a segment image is not read by its first update
+    cells = float(np.prod([n + 2 * wl.pad for n in (20, 18, 22)]))
+    assert s["bytes_adjoint"] == pytest.approx(cells * 2 * 3 * per_cell, rel=1e-12)
