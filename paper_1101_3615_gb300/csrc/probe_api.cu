@@ -50,6 +50,7 @@ probe_status fail(probe_t h, probe_status st, const std::string& msg) {
 
 probe_status cuda_fail(probe_t h, cudaError_t e, const char* what) {
     const probe_status st = (e == cudaErrorMemoryAllocation) ? PROBE_ERR_OOM : PROBE_ERR_CUDA;
+    if (st == PROBE_ERR_OOM) cudaGetLastError();  // reported here, not by the caller's next CUDA call
     return fail(h, st, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
@@ -1761,6 +1762,7 @@ extern "C" probe_status probe_create(probe_t* out, const probe_grid* g, const fl
 
     auto cuda_bad = [&](cudaError_t e, const char* what) {
         std::string m = std::string(what) + ": " + cudaGetErrorString(e);
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();
         probe_destroy(h);
         return fail(nullptr, e == cudaErrorMemoryAllocation ? PROBE_ERR_OOM : PROBE_ERR_CUDA, m);
     };

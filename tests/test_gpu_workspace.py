@@ -1,0 +1,68 @@
+"""Device memory of a handle's workspace: what a call reserves, and calls where memory is short.
+
+Free memory is read from the device; "short" is made by holding most of it in a tensor.  Sizes are chosen
+so that the routes differ by tens of megabytes (reservations) or gigabytes (short memory).
+"""
+import contextlib
+import gc
+
+import numpy as np
+import pytest
+
+from workloads import mini_config
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+MB = 1 << 20
+
+
+def probe_of(wl, **kw):
+    from paper_1101_3615_gb300 import Probe
+    return Probe(wl.m0, wl.h, wl.dt, wl.nt, wl.pad, wl.src, wl.rec, wl.wavelet, **kw)
+
+
+def workload(shape, nt, ns, nb, pad=20):
+    rng = np.random.default_rng(2)
+    wl = mini_config(2, shape=shape, nt=nt, ns=1, pad=pad, p=1)
+    wl.src = np.stack([np.full(ns, 2), rng.integers(0, shape[1], ns)], 1).astype(np.int32)
+    wl.trials = (rng.standard_normal((nb,) + tuple(shape)) * 0.05 * wl.m0.mean()).astype(np.float32)
+    return wl
+
+
+def free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+@contextlib.contextmanager
+def only(leave):
+    """Most of the device memory held, `leave` bytes of it free."""
+    gc.collect()
+    torch.cuda.empty_cache()
+    held = torch.empty(free() - leave, dtype=torch.uint8, device="cuda")
+    try:
+        yield
+    finally:
+        del held
+        torch.cuda.empty_cache()
+
+
+def rel(a, b):
+    return float((a.double() - b.double()).norm() / b.double().norm())
+
+
+def test_out_of_memory_is_reported_once(cuda_device):
+    """The status of the call that ran out; what comes next finds no error of it."""
+    from paper_1101_3615_gb300 import ProbeError
+    wl = workload((200, 200), 201, 64, 4)
+    y = torch.tensor(wl.trials, device=cuda_device)
+    p = probe_of(wl, ckpt_stride=100)
+    p.set_option("shot_wave", 64)
+    with only(512 * MB):
+        with pytest.raises(ProbeError) as ei:
+            p.apply_H(y)
+        assert ei.value.status == -3
+        z = y + 1.0
+    p.apply_H(y)
+    assert float((z - y).mean()) == pytest.approx(1.0)
