@@ -184,7 +184,6 @@ void free_ws(Workspace& w) {
 // planes (3D) that hold receivers.
 long long inj_block(probe_t h) { return (long long)h->nband * (h->ndim == 3 ? (long long)h->Ny * h->P : h->P); }
 
-// Bytes per resident shot and fixed bytes of a job with nb trials.
 bool use_history(probe_t h, int with_ckpt) { return with_ckpt && h->opt_dtt_history && h->ndim == 2; }
 
 // Levels of one launch of the resident kernels.  A call with checkpoints: the checkpoint stride.
@@ -219,36 +218,52 @@ int dtt_slots_2d(probe_t h, int with_ckpt, int history, int res) {
 // rather than the one-barrier-per-plane kernel or the shot-cluster kernel.
 bool adj3d_ws(probe_t h) { return h->ndim == 3 && h->pipe_adj != 0 && !(h->opt_cluster3d & 2); }
 
-void ws_bytes(probe_t h, int nb, int with_ckpt, int with_data, int res, double* per_shot, double* fixed) {
-    const double F4 = (double)h->F * 4.0;
-    double ps = 2 * F4 + 2.0 * nb * F4;
-    if (h->ndim == 2) ps += 4 * F4 + 4.0 * nb * F4;  // four-level states of the time-blocked forward
-    if (use_history(h, with_ckpt))
-        ps += (double)(h->nt - 1) * F4;
-    else if (with_ckpt)
-        ps += (double)h->nck * ckpt_bytes_per_shot(h->snap, h->F) + (res ? 2.0 : 1.0) * h->K * F4 + 16.0 * h->nck;
-    else if (h->ndim == 3)
-        ps += 2.0 * F4;  // Dtt u^n of two steps (Born source)
-    else if (res)
-        ps += 2.0 * res_seg(h, 0) * F4;
-    if (with_data) ps += (double)nb * h->nt * h->nr * 4.0;
-    if (h->ndim == 3 && with_ckpt) {
-        ps += 2.0 * nb * F4;  // per-shot images + compensation
-        if ((h->opt_cluster3d & 2) || adj3d_ws(h)) ps += (double)h->K * nb * inj_block(h) * 4.0;  // injection of one segment
-        if (!(h->opt_cluster3d & 2) && h->kahan) ps += (double)nb * F4;                          // segment images
+// Device arrays of a workspace for W resident shots and nb trials, in bytes: what ensure_ws allocates
+// and plan_wave counts.
+struct WsBytes {
+    size_t u, f, dm, data, ckpt, scales, absmax, dtt, img, comp, seg, s_tmp, src, inj, u4, f4;
+    double total() const {
+        return (double)u + f + dm + data + ckpt + scales + absmax + dtt + img + comp + seg + s_tmp + src + inj + u4 + f4;
     }
-    *per_shot = ps;
-    *fixed = nb * F4 + 2.0 * F4 * nb + F4;  // dm, one image group, s_tmp
+};
+WsBytes ws_bytes(probe_t h, int W, int nb, int with_ckpt, int with_data, int res) {
+    const size_t F4 = (size_t)h->F * 4, w = (size_t)W, b = (size_t)std::max(nb, 1);
+    const bool two = h->ndim == 2, history = use_history(h, with_ckpt), store = with_ckpt && !history;
+    WsBytes s{};
+    s.u = w * 2 * F4;
+    s.f = w * b * 2 * F4;
+    s.dm = b * F4;
+    if (with_data) s.data = w * nb * h->nt * h->nr * 4;
+    if (store) {
+        s.ckpt = h->nck * w * ckpt_bytes_per_shot(h->snap, h->F);
+        s.scales = h->nck * w * 2 * 4;
+        s.absmax = w * 2 * 4;
+    }
+    const int slots = two ? dtt_slots_2d(h, with_ckpt, history, res) : (with_ckpt ? h->K : 2);
+    if (!two || slots > 1 || with_ckpt) s.dtt = w * slots * F4;
+    s.img = s.comp = w * b * F4;  // image groups of one shot: any group size fits
+    if (!two && with_ckpt && h->kahan && !(h->opt_cluster3d & 2)) s.seg = w * b * F4;
+    s.s_tmp = F4;
+    s.src = w * 3 * 4;
+    // one segment of adjoint injection (two for the resident kernels)
+    if (with_ckpt && h->nband > 0 && (two || (h->opt_cluster3d & 2) || adj3d_ws(h)))
+        s.inj = (two && res && !history ? 2 : 1) * h->K * w * b * inj_block(h) * 4;
+    if (two) {  // four-level states of the time-blocked forward
+        s.u4 = w * 4 * F4;
+        s.f4 = w * b * 4 * F4;
+    }
+    return s;
 }
 
 int plan_wave(probe_t h, int nb, int with_ckpt, int with_data, int res) {
     if (h->opt_shot_wave > 0) return std::min(h->opt_shot_wave, h->ns);
-    double ps, fx;
-    ws_bytes(h, nb, with_ckpt, with_data, res, &ps, &fx);
+    const double one = ws_bytes(h, 1, nb, with_ckpt, with_data, res).total();
+    const double per_shot = ws_bytes(h, 2, nb, with_ckpt, with_data, res).total() - one;
     size_t freeb = 0, totb = 0;
     cudaMemGetInfo(&freeb, &totb);
-    const double budget = 0.80 * (double)freeb + (double)h->ws.bytes;
-    int W = std::max(1, std::min((int)std::floor((budget - fx) / ps), h->ns));
+    // (the same with the workspace allocated as before it: a call plans what the one before it did)
+    const double budget = 0.80 * ((double)freeb + (double)h->ws.bytes);
+    int W = 1 + (int)std::max(0.0, std::min(std::floor((budget - one) / per_shot), h->ns - 1.0));
     // equal waves: the fewest waves that fit, with the shots spread evenly over them (so that the
     // last wave is not a remainder of one or two shots)
     const int nwaves = (h->ns + W - 1) / W;
@@ -298,7 +313,6 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, i
         w.groups >= G && w.tm_tile_z == h->tile_z && w.W == W && w.nb == nb && w.history == history)
         return PROBE_OK;
     free_ws(w);
-    const long long F = h->F;
     auto alloc = [&](void** p, size_t bytes) -> probe_status {
         if (bytes == 0) return PROBE_OK;
         cudaError_t e = cudaMalloc(p, bytes);
@@ -309,40 +323,30 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, i
         w.bytes += bytes;
         return PROBE_OK;
     };
-    TRY(alloc((void**)&w.u, (size_t)W * 2 * F * 4));
-    TRY(alloc((void**)&w.f, (size_t)W * std::max(nb, 1) * 2 * F * 4));
-    TRY(alloc((void**)&w.dm, (size_t)std::max(nb, 1) * F * 4));
-    if (with_data) TRY(alloc((void**)&w.data, (size_t)W * nb * h->nt * h->nr * 4));
-    if (history) {
-        TRY(alloc((void**)&w.dtt, (size_t)W * (h->nt - 1) * F * 4));  // Dtt u^n of every step
-    } else if (with_ckpt) {
-        TRY(alloc(&w.ckpt, (size_t)h->nck * W * ckpt_bytes_per_shot(h->snap, F)));
-        TRY(alloc((void**)&w.scales, (size_t)h->nck * W * 2 * 4));
-        TRY(alloc((void**)&w.absmax, (size_t)W * 2 * 4));
-        TRY(alloc((void**)&w.dtt, (size_t)W * (h->ndim == 2 ? slots2 : h->K) * F * 4));
-    } else if (h->ndim == 3) {
-        TRY(alloc((void**)&w.dtt, (size_t)W * 2 * F * 4));  // Dtt u^n of two steps (Born source)
-    } else if (slots2 > 1) {
-        TRY(alloc((void**)&w.dtt, (size_t)W * slots2 * F * 4));
-    }
-    TRY(alloc((void**)&w.img, (size_t)G * std::max(nb, 1) * F * 4));
-    TRY(alloc((void**)&w.comp, (size_t)G * std::max(nb, 1) * F * 4));
-    if (h->ndim == 3 && with_ckpt && h->kahan && !(h->opt_cluster3d & 2)) {
-        TRY(alloc((void**)&w.seg, (size_t)W * std::max(nb, 1) * F * 4));
-        CK(h, cudaMemset(w.seg, 0, (size_t)W * std::max(nb, 1) * F * 4));  // pitch columns stay zero
-    }
-    TRY(alloc((void**)&w.s_tmp, (size_t)F * 4));
-    TRY(alloc((void**)&w.src_wave, (size_t)W * 3 * 4));
-    // one segment of adjoint injection (two for the resident kernels)
-    if (with_ckpt && h->nband > 0 && (h->ndim == 2 || (h->opt_cluster3d & 2) || adj3d_ws(h)))
-        TRY(alloc((void**)&w.inj, (size_t)(slots2 > h->K && !history ? 2 : 1) * h->K * W * std::max(nb, 1) *
-                                      inj_block(h) * 4));
+    const WsBytes s = ws_bytes(h, W, nb, with_ckpt, with_data, res);
+    TRY(alloc((void**)&w.u, s.u));
+    TRY(alloc((void**)&w.f, s.f));
+    TRY(alloc((void**)&w.dm, s.dm));
+    TRY(alloc((void**)&w.data, s.data));
+    TRY(alloc(&w.ckpt, s.ckpt));
+    TRY(alloc((void**)&w.scales, s.scales));
+    TRY(alloc((void**)&w.absmax, s.absmax));
+    TRY(alloc((void**)&w.dtt, s.dtt));  // Dtt u^n of every step, of one or two segments, 3D forward: of two steps
+    TRY(alloc((void**)&w.img, s.img));
+    TRY(alloc((void**)&w.comp, s.comp));
+    TRY(alloc((void**)&w.seg, s.seg));
+    if (w.seg) CK(h, cudaMemset(w.seg, 0, s.seg));  // pitch columns stay zero
+    TRY(alloc((void**)&w.s_tmp, s.s_tmp));
+    TRY(alloc((void**)&w.src_wave, s.src));
+    TRY(alloc((void**)&w.inj, s.inj));
+    TRY(alloc((void**)&w.u4, s.u4));
+    TRY(alloc((void**)&w.f4, s.f4));
     // field planes must read as zero outside what the kernels write
-    CK(h, cudaMemset(w.u, 0, (size_t)W * 2 * F * 4));
-    CK(h, cudaMemset(w.f, 0, (size_t)W * std::max(nb, 1) * 2 * F * 4));
+    CK(h, cudaMemset(w.u, 0, s.u));
+    CK(h, cudaMemset(w.f, 0, s.f));
     w.history = history;
     w.dtt_slots = h->ndim == 2 ? slots2 : (with_ckpt ? h->K : 2);
-    if (w.dtt) CK(h, cudaMemset(w.dtt, 0, (size_t)W * w.dtt_slots * F * 4));
+    if (w.dtt) CK(h, cudaMemset(w.dtt, 0, s.dtt));
     w.W = W;
     w.nb = nb;
     w.with_ckpt = with_ckpt;
@@ -354,10 +358,8 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, i
         TRY(encode_ws_maps(h, w.mf, h->ws_rows));
         TRY(encode_ws_maps(h, w.ma, h->ws_rows_adj));
         // four-level states of the time-blocked forward (zero: levels -1 and 0 start at rest)
-        TRY(alloc((void**)&w.u4, (size_t)W * 4 * F * 4));
-        TRY(alloc((void**)&w.f4, (size_t)W * std::max(nb, 1) * 4 * F * 4));
-        CK(h, cudaMemset(w.u4, 0, (size_t)W * 4 * F * 4));
-        CK(h, cudaMemset(w.f4, 0, (size_t)W * std::max(nb, 1) * 4 * F * 4));
+        CK(h, cudaMemset(w.u4, 0, s.u4));
+        CK(h, cudaMemset(w.f4, 0, s.f4));
         TRY(encode_box(h, &w.tm_u4h, w.u4, W * 4, kTX + 16, 32));
         TRY(encode_box(h, &w.tm_u4e, w.u4, W * 4, kTX + 8, 24));
         TRY(encode_box(h, &w.tm_f4h, w.f4, W * std::max(nb, 1) * 4, kTX + 16, 32));

@@ -52,6 +52,28 @@ def rel(a, b):
     return float((a.double() - b.double()).norm() / b.double().norm())
 
 
+@pytest.mark.parametrize("pipeline", [None, 2])
+def test_planned_waves_fit_with_receivers_on_every_row(cuda_device, pipeline):
+    """The receiver injection of a segment (200 bands) is most of the workspace."""
+    wl = workload((200, 200), 201, 64, 4)
+    wl.rec = np.stack([np.arange(200), np.full(200, 100)], 1).astype(np.int32)
+    y = torch.tensor(wl.trials, device=cuda_device)
+
+    def handle():
+        p = probe_of(wl, ckpt_stride=100)
+        if pipeline:
+            p.set_option("pipeline", pipeline)
+        return p
+
+    p = handle()
+    ref = p.apply_H(y)
+    assert p.stats()["shot_wave"] == 64
+    p = handle()
+    with only(4096 * MB):
+        assert rel(p.apply_H(y), ref) < 1e-6
+        assert p.stats()["shot_wave"] < 64
+
+
 def test_out_of_memory_is_reported_once(cuda_device):
     """The status of the call that ran out; what comes next finds no error of it."""
     from paper_1101_3615_gb300 import ProbeError
