@@ -2176,9 +2176,10 @@ void add_counts(probe_stats& s, const Job& jb, FwdKind kind, bool need_ckpt, boo
 }
 
 // Run one operator on one model.  dm: device [nb][n]; data_user: device [nb][ns][nt][nr] (F / F*)
-// or [ns][nt][nr] (nonlinear / gradient); img_out: device [nb][n].
+// or [ns][nt][nr] (nonlinear / gradient); img_out: device [nb][n]; m: device [n], the model of the
+// nonlinear map and its gradient (null: the background model).
 probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in, float* data_out,
-                    float* img_out, int nb, const float* s, cudaStream_t st) {
+                    float* img_out, int nb, const float* m, cudaStream_t st) {
     const bool need_ckpt = (op == OP_FADJ || op == OP_H || op == OP_GRAD);
     const bool need_data = (op == OP_H);
     const int nbw = (op == OP_NONLIN || op == OP_GRAD) ? 1 : nb;
@@ -2196,6 +2197,13 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
         cudaError_t e = launch_embed(dm_dev, w.dm, nb, h->nz, h->nx, h->ny, h->pad, h->Nz, h->Nx, h->Ny, h->P,
                                      h->F, 1.0f, st);
         if (e != cudaSuccess) return cuda_fail(h, e, "embed dm");
+    }
+    const float* s = h->d_s0;
+    if (m) {  // positivity is the caller's responsibility; non-finite values are caught by the output check
+        cudaError_t e = launch_make_s(m, h->d_m0, w.s_tmp, h->nz, h->ny, h->nx, h->pad, h->P, h->F, h->Nz, h->Ny, h->Nx,
+                                      (float)(h->dt * h->dt), st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "make s");
+        s = w.s_tmp;
     }
     const int nwaves = (h->ns + W - 1) / W;
     const int nev = 3 + 2 * h->nck + 2;
@@ -2369,7 +2377,7 @@ extern "C" probe_status probe_apply_F(probe_t h, const float* dm, float* d, int 
         TRY(ensure_buf(h, h->stage_out, nd * 4));
         dd = (float*)h->stage_out.p;
     }
-    TRY(run_op(h, OP_F, dmd, nullptr, dd, nullptr, nb, h->d_s0, st));
+    TRY(run_op(h, OP_F, dmd, nullptr, dd, nullptr, nb, nullptr, st));
     TRY(finish_call(h, st, hin || hout, dd, (long long)nd));
     if (hout) {
         CK(h, cudaMemcpyAsync(d, dd, nd * 4, cudaMemcpyDeviceToHost, st));
@@ -2394,7 +2402,7 @@ extern "C" probe_status probe_apply_Fadj(probe_t h, const float* d, float* img, 
         TRY(ensure_buf(h, h->stage_out, (size_t)nb * h->nmodel * 4));
         io = (float*)h->stage_out.p;
     }
-    TRY(run_op(h, OP_FADJ, nullptr, dd, nullptr, io, nb, h->d_s0, st));
+    TRY(run_op(h, OP_FADJ, nullptr, dd, nullptr, io, nb, nullptr, st));
     TRY(finish_call(h, st, hin || hout, io, (long long)nb * h->nmodel));
     if (hout) {
         CK(h, cudaMemcpyAsync(img, io, (size_t)nb * h->nmodel * 4, cudaMemcpyDeviceToHost, st));
@@ -2418,7 +2426,7 @@ extern "C" probe_status probe_apply_H(probe_t h, const float* dm, float* Hdm, in
         TRY(ensure_buf(h, h->stage_out, (size_t)nb * h->nmodel * 4));
         o = (float*)h->stage_out.p;
     }
-    TRY(run_op(h, OP_H, dmd, nullptr, nullptr, o, nb, h->d_s0, st));
+    TRY(run_op(h, OP_H, dmd, nullptr, nullptr, o, nb, nullptr, st));
     TRY(finish_call(h, st, hin || hout, o, (long long)nb * h->nmodel));
     if (hout) {
         CK(h, cudaMemcpyAsync(Hdm, o, (size_t)nb * h->nmodel * 4, cudaMemcpyDeviceToHost, st));
@@ -2441,13 +2449,7 @@ extern "C" probe_status probe_forward_nonlinear(probe_t h, const float* m, float
         TRY(ensure_buf(h, h->stage_out, nd * 4));
         dd = (float*)h->stage_out.p;
     }
-    const int fits = res_fits(h, 0, 0);
-    TRY(ensure_ws(h, plan_wave(h, 1, 0, 0, fits), 1, 0, 0, fits));
-    // positivity of m is the caller's responsibility; non-finite values are caught by the output check
-    cudaError_t e = launch_make_s(md, h->d_m0, h->ws.s_tmp, h->nz, h->ny, h->nx, h->pad, h->P, h->F, h->Nz, h->Ny,
-                                  h->Nx, (float)(h->dt * h->dt), st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "make s");
-    TRY(run_op(h, OP_NONLIN, nullptr, nullptr, dd, nullptr, 1, h->ws.s_tmp, st));
+    TRY(run_op(h, OP_NONLIN, nullptr, nullptr, dd, nullptr, 1, md, st));
     TRY(finish_call(h, st, hin || hout, dd, (long long)nd));
     if (hout) {
         CK(h, cudaMemcpyAsync(d, dd, nd * 4, cudaMemcpyDeviceToHost, st));
@@ -2483,16 +2485,7 @@ extern "C" probe_status probe_gradient(probe_t h, const float* m, const float* r
     }
     probe_status st_ = PROBE_OK;
     do {
-        const int fits = res_fits(h, 1, 0);
-        st_ = ensure_ws(h, plan_wave(h, 1, 1, 0, fits), 1, 1, 0, fits);
-        if (st_ != PROBE_OK) break;
-        cudaError_t e = launch_make_s(md, h->d_m0, h->ws.s_tmp, h->nz, h->ny, h->nx, h->pad, h->P, h->F, h->Nz,
-                                      h->Ny, h->Nx, (float)(h->dt * h->dt), st);
-        if (e != cudaSuccess) {
-            st_ = cuda_fail(h, e, "make s");
-            break;
-        }
-        st_ = run_op(h, OP_GRAD, nullptr, rd, nullptr, go, 1, h->ws.s_tmp, st);
+        st_ = run_op(h, OP_GRAD, nullptr, rd, nullptr, go, 1, md, st);
         if (st_ != PROBE_OK) break;
         st_ = finish_call(h, st, true, go, h->nmodel);
         if (st_ != PROBE_OK) break;

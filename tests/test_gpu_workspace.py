@@ -88,3 +88,18 @@ def test_out_of_memory_is_reported_once(cuda_device):
         z = y + 1.0
     p.apply_H(y)
     assert float((z - y).mean()) == pytest.approx(1.0)
+
+
+def test_gradient_in_planned_waves(cuda_device):
+    """The model of a gradient is prepared in the workspace that its sweeps run in, whatever wave is planned."""
+    wl = workload((100, 100), 401, 64, 1)
+    m = torch.tensor(wl.m0, device=cuda_device) * 1.01
+    p = probe_of(wl, ckpt_stride=400)
+    d = p.forward_nonlinear(m)
+    ref = p.gradient(m, d)
+    p = probe_of(wl, ckpt_stride=400)
+    with only(3072 * MB):
+        for _ in range(2):
+            assert rel(p.gradient(m, d), ref) < 1e-6
+            assert p.stats()["shot_wave"] < 64
+        assert rel(p.forward_nonlinear(m), d) < 1e-6
