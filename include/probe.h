@@ -199,8 +199,9 @@ typedef struct {
     int pipeline_rows;           /* rows per thread of the pipelined forward kernels (0: not pipelined) */
     int pipeline_rows_adjoint;   /* rows per thread of the pipelined adjoint kernel */
     int time_block;              /* 2D Born forward and recompute: time levels per launch (1 or 2;
-                                    cluster-resident kernels: the checkpoint stride, up to twice it
-                                    for calls without checkpoints) */
+                                    cluster-resident kernels: the checkpoint stride, in calls without
+                                    checkpoints twice it where the Dtt planes stay in L2, half of it in a
+                                    workspace made for the one-level adjoint) */
     int planes_3d;               /* 3D: z planes marched by one CTA (0 for 2D) */
     int pipeline_incident;       /* 3D: as pipeline_forward, for the incident step (forward and
                                     recompute; pipeline_forward then names the Born step's) */

@@ -23,6 +23,7 @@ struct Workspace {
     int W = 0, nb = 0, with_ckpt = 0, with_data = 0, groups = 0;
     int history = 0;          // Dtt u^n kept for every step (no checkpoints)
     int dtt_slots = 0;        // Dtt planes per shot
+    int inj_sets = 1;         // segments of adjoint injection
     size_t bytes = 0;
     float* u = nullptr;       // [W][2][F]
     float* f = nullptr;       // [W][nb][2][F]
@@ -34,13 +35,13 @@ struct Workspace {
     void* ckpt = nullptr;     // [nck][W][2][F] (fp32 or 16-bit)
     float* scales = nullptr;  // [nck][W*2]
     float* absmax = nullptr;  // [W*2]
-    float* dtt = nullptr;     // [W][K][F]
+    float* dtt = nullptr;     // [W][dtt_slots][F]
     float* img = nullptr;     // [groups][nb][F]
     float* seg = nullptr;     // 3D one-field adjoint with Kahan: plain FP32 image of one checkpoint segment
     float* comp = nullptr;
     float* s_tmp = nullptr;   // [F]
     int* src_wave = nullptr;  // [W][2] padded sources of the wave
-    float* inj = nullptr;     // [K][W][nb][nband][P] adjoint injection of one segment (2D)
+    float* inj = nullptr;     // [inj_sets][K][W][nb][nband][P] adjoint injection of a segment (2D)
     CUtensorMap tm_u, tm_f;
     // pipelined kernels: halo and plain boxes for tiles of 64 x 16 rows, one set for the
     // forward kernels and one for the adjoint (their row counts are chosen separately)

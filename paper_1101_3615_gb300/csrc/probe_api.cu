@@ -206,12 +206,13 @@ bool res_fits(probe_t h, int with_ckpt, int born) {
     return fits(RES_INC) && (!born || fits(RES_BORN)) && (!with_ckpt || fits(RES_ADJ));
 }
 
-// Dtt planes per shot of a 2D workspace: the history; two segments for the resident kernels (one
-// being read while the next is written); one checkpoint segment; none (1, unallocated).
+// Dtt planes per shot of a 2D workspace: the history; two segments for calls that run Born or adjoint
+// fields on the resident kernels (res; one being read while the next is written); one checkpoint segment
+// (of two planes at least, so that it also serves resident forward calls); none (1, unallocated).
 int dtt_slots_2d(probe_t h, int with_ckpt, int history, int res) {
     if (history) return h->nt - 1;
     if (res) return 2 * res_seg(h, with_ckpt);
-    return with_ckpt ? h->K : 1;
+    return with_ckpt ? std::max(h->K, 2) : 1;
 }
 
 // 3D adjoint on the producer-warp kernel (receiver injection from a per-segment band buffer)
@@ -247,7 +248,7 @@ WsBytes ws_bytes(probe_t h, int W, int nb, int with_ckpt, int with_data, int res
     s.src = w * 3 * 4;
     // one segment of adjoint injection (two for the resident kernels)
     if (with_ckpt && h->nband > 0 && (two || (h->opt_cluster3d & 2) || adj3d_ws(h)))
-        s.inj = (two && res && !history ? 2 : 1) * h->K * w * b * inj_block(h) * 4;
+        s.inj = (two && res ? 2 : 1) * h->K * w * b * inj_block(h) * 4;
     if (two) {  // four-level states of the time-blocked forward
         s.u4 = w * 4 * F4;
         s.f4 = w * b * 4 * F4;
@@ -308,8 +309,11 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, i
     const int G = W;  // image groups for the smallest shot group: any group size fits
     const int history = use_history(h, with_ckpt) ? 1 : 0;
     const int slots2 = h->ndim == 2 ? dtt_slots_2d(h, with_ckpt, history, res) : 0;
-    // (a workspace with checkpoint segments serves calls without them, in shorter launches)
-    if (w.u && (h->ndim == 3 || w.dtt_slots >= std::min(slots2, 2 * h->K)) && w.W >= W && w.nb >= nb && w.with_ckpt >= with_ckpt && w.with_data >= with_data &&
+    // a workspace with checkpoint segments serves calls without them too, in launches of half its planes: calls
+    // with and without in turn keep it
+    const int need = !with_ckpt && w.with_ckpt ? std::min(slots2, 2) : slots2;
+    const int inj_sets = h->ndim == 2 && with_ckpt && res ? 2 : 1;
+    if (w.u && (h->ndim == 3 || w.dtt_slots >= need) && w.inj_sets >= inj_sets && w.W >= W && w.nb >= nb && w.with_ckpt >= with_ckpt && w.with_data >= with_data &&
         w.groups >= G && w.tm_tile_z == h->tile_z && w.W == W && w.nb == nb && w.history == history)
         return PROBE_OK;
     free_ws(w);
@@ -345,6 +349,7 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, i
     CK(h, cudaMemset(w.u, 0, s.u));
     CK(h, cudaMemset(w.f, 0, s.f));
     w.history = history;
+    w.inj_sets = inj_sets;
     w.dtt_slots = h->ndim == 2 ? slots2 : (with_ckpt ? h->K : 2);
     if (w.dtt) CK(h, cudaMemset(w.dtt, 0, s.dtt));
     w.W = W;
@@ -933,9 +938,10 @@ void fill_res(const Job& jb, ResParams2D& p) {
 }
 
 // The incident field's chain (checkpoint store or restore, levels of a segment) runs on the second
-// stream, the Born / adjoint chain on the call's: segment i uses Dtt slots (i & 1) K .. + K - 1, the
-// incident launch i + 2 waits for the last reader of its slots.  Each chain alone leaves SMs idle.
-probe_status run_forward_res(Sweep& sw, Job& jb, const ResSet& rs, FwdKind kind, bool ckpt) {
+// stream, the Born / adjoint chain on the call's: segment i (seg levels; with checkpoints the
+// stride) uses Dtt slots (i & 1) seg .. + seg - 1, the incident launch i + 2 waits for the last reader of its
+// slots.  Each chain alone leaves SMs idle.
+probe_status run_forward_res(Sweep& sw, Job& jb, const ResSet& rs, FwdKind kind, bool ckpt, int seg) {
     probe_t h = jb.h;
     Workspace& w = h->ws;
     cudaStream_t st = sw.st;
@@ -964,7 +970,6 @@ probe_status run_forward_res(Sweep& sw, Job& jb, const ResSet& rs, FwdKind kind,
         CK(h, cudaEventRecord(h->ov_inc[0], st));
         CK(h, cudaStreamWaitEvent(su, h->ov_inc[0], 0));
     }
-    const int seg = born ? std::min(res_seg(h, ckpt), w.dtt_slots / 2) : res_seg(h, ckpt);
     for (int n = 0, i = 0; n < h->nt - 1; n += seg, ++i) {
         const int T = std::min(seg, h->nt - 1 - n), set = i & 1;
         if (born && i >= 2) CK(h, cudaStreamWaitEvent(su, h->ov_born[set], 0));
@@ -1111,9 +1116,9 @@ double one_level_us(double fwd, double adj) { return 7.5 + 2.3 * fwd + (adj > 0 
 // shots, 1 and 4 trials, they take 0.20 to 0.92 of the one-level kernels' time.  Forward only, where
 // the estimate is below the one-level kernels': few fields 0.39 to 0.6 of their time, equal at about
 // six million cells in flight, and up to 1.5 beyond (325 x 445, 64 shots, 4 trials: one cluster of 16
-// SMs at a time holds a field, 112 of 152 SMs), where the one-level kernels stay.
-const ResSet& res_set(probe_t h, FwdKind kind, bool adjoint, int W, int nb) {
-    const std::vector<long long> key = {(long long)kind, (long long)adjoint, W, nb, h->user_fixed, h->user_tblock,
+// SMs at a time holds a field, 112 of 152 SMs), where the one-level kernels stay.  T: levels per launch.
+const ResSet& res_set(probe_t h, FwdKind kind, bool adjoint, int W, int nb, int T) {
+    const std::vector<long long> key = {(long long)kind, (long long)adjoint, W, nb, T, h->user_fixed, h->user_tblock,
                                         h->opt_tile_z, h->opt_dtt_history, h->opt_autotune};
     for (const ResSet& r : h->res_sets)
         if (r.key == key) return r;
@@ -1121,7 +1126,6 @@ const ResSet& res_set(probe_t h, FwdKind kind, bool adjoint, int W, int nb) {
     r.key = key;
     const bool born = kind == FWD_BORN, kh = h->kahan != 0;
     if (res_fits(h, adjoint, born)) {
-        const int T = res_seg(h, adjoint);
         const std::vector<ResPlan> inc = plan_res2d(RES_INC, kh, h->Nz, h->Nx, h->pad, T);
         std::vector<ResPlan> bo, ad;
         if (born) bo = plan_res2d(RES_BORN, kh, h->Nz, h->Nx, h->pad, T);
@@ -2184,11 +2188,20 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
     const bool need_data = (op == OP_H);
     const int nbw = (op == OP_NONLIN || op == OP_GRAD) ? 1 : nb;
     const FwdKind kind = (op == OP_F || op == OP_H) ? FWD_BORN : (op == OP_NONLIN) ? FWD_INCIDENT_SAMPLE : FWD_INCIDENT;
-    const int fits = res_fits(h, need_ckpt, kind == FWD_BORN);
-    const int W = plan_wave(h, nbw, need_ckpt, need_data, fits);
-    TRY(ensure_ws(h, W, nbw, need_ckpt, need_data, fits));
+    const bool res_dtt = need_ckpt || kind == FWD_BORN;  // on the resident kernels: two segments of Dtt
+    const int T = res_seg(h, need_ckpt);
+    ResSet rs;
+    int W = 0;
+    if (res_fits(h, need_ckpt, kind == FWD_BORN)) {
+        W = plan_wave(h, nbw, need_ckpt, need_data, res_dtt);
+        rs = res_set(h, kind, need_ckpt, W, nbw, T);
+    }
+    if (!rs.use) W = plan_wave(h, nbw, need_ckpt, need_data, 0);
+    TRY(ensure_ws(h, W, nbw, need_ckpt, need_data, rs.use && res_dtt));
     Workspace& w = h->ws;
-    const ResSet rs = h->ndim == 2 ? res_set(h, kind, need_ckpt, W, nbw) : ResSet();
+    // levels per launch in this workspace; the estimate again where it has fewer planes
+    const int seg = rs.use && kind == FWD_BORN ? std::min(T, w.dtt_slots / 2) : T;
+    if (seg < T) rs = res_set(h, kind, need_ckpt, W, nbw, seg);
     int G = 0;
     reset_stats(h);
     h->stats.shot_wave = W;
@@ -2278,7 +2291,7 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
             }
             h->stats.pipeline_rows = piped ? h->ws_rows : 0;
             h->stats.pipeline_rows_adjoint = piped ? h->ws_rows_adj : 0;
-            h->stats.time_block = rs.use ? res_seg(h, need_ckpt) : (h->ndim == 2 && h->tile_z == kPipeTZ && w.u4) ? h->opt_tblock : 1;
+            h->stats.time_block = rs.use ? seg : (h->ndim == 2 && h->tile_z == kPipeTZ && w.u4) ? h->opt_tblock : 1;
             if (need_ckpt) {
                 CK(h, cudaMemsetAsync(w.img, 0, (size_t)G * nbw * h->F * 4, st));
                 CK(h, cudaMemsetAsync(w.comp, 0, (size_t)G * nbw * h->F * 4, st));
@@ -2311,7 +2324,7 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
                 else
                     TRY(prepare_sweep(sw2, h, ss));
                 record(h, 0, ss);
-                TRY(rs.use ? run_forward_res(sw2, sw2.jobs[0], rs, kind, need_ckpt) : run_forward(sw2, kind, need_ckpt));
+                TRY(rs.use ? run_forward_res(sw2, sw2.jobs[0], rs, kind, need_ckpt, seg) : run_forward(sw2, kind, need_ckpt));
                 record(h, 1, ss);
                 int ev = 2;
                 if (need_ckpt) TRY(rs.use ? run_adjoint_res(sw2, sw2.jobs[0], rs, h, &ev) : run_adjoint(sw2));
@@ -2534,7 +2547,7 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
     if (res) {  // the resident kernels take the models in turn, the one-level kernels all at once
         double us = 0.0, fwd = 0.0, rev = 0.0;
         for (int k = 0; k < nmodels; ++k) {
-            rss[k] = res_set(models[k], FWD_BORN, true, models[k]->ns, nb[k]);
+            rss[k] = res_set(models[k], FWD_BORN, true, models[k]->ns, nb[k], h0->K);
             us += rss[k].us;
             fwd += rss[k].fwd;
             rev += rss[k].rev;
@@ -2619,7 +2632,7 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
         if (res) {  // model after model
             sw2.st = ss;
             record(h0, 0, ss);
-            for (int k = 0; k < nmodels; ++k) TRY(run_forward_res(sw2, sw2.jobs[k], rss[k], FWD_BORN, true));
+            for (int k = 0; k < nmodels; ++k) TRY(run_forward_res(sw2, sw2.jobs[k], rss[k], FWD_BORN, true, h0->K));
             record(h0, 1, ss);
             int ev = 2;
             for (int k = 0; k < nmodels; ++k) TRY(run_adjoint_res(sw2, sw2.jobs[k], rss[k], h0, &ev));

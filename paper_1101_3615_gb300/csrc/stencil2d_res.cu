@@ -1,9 +1,9 @@
 // Cluster-resident 2D time stepping (sm_103a): many time levels per launch.
 //
 // A field whose grid fits the shared memory of one thread-block cluster stays there for a whole
-// checkpoint segment.  The cluster's CTAs own contiguous strips of grid rows (full width); a launch
-// loads the two levels of the state, the medium and the pointwise operands once, advances up to
-// ceil(sqrt(nt)) levels, and writes the two last levels back.  Per level a CTA computes its rows
+// segment of time levels.  The cluster's CTAs own contiguous strips of grid rows (full width); a launch
+// loads the two levels of the state, the medium and the pointwise operands once, advances a segment (the
+// checkpoint stride; up to twice that in calls without checkpoints), and writes the two last levels back.  Per level a CTA computes its rows
 // from the level in shared memory, writes the new level over the older one, and stores its first and
 // last four rows into the neighbouring CTAs' halo rows as well (asynchronous distributed-shared-memory
 // stores that complete on the neighbour's mbarrier, so data and signal travel together and no store

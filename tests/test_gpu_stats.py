@@ -78,6 +78,19 @@ def test_resident_group_times_cover_every_model(cuda_device):
     assert late < 1.5 * max(single)
 
 
+def test_resident_time_block_is_the_launched_segment(cuda_device):
+    wl = workload((50, 60), 200, 2, 2)
+    y = torch.tensor(wl.trials, device=cuda_device)
+    fresh, used = probe_of(wl), probe_of(wl)
+    used.apply_H(y)                       # a workspace with checkpoint segments: shorter launches
+    ref = fresh.apply_F(y)
+    assert torch.equal(used.apply_F(y), ref)
+    for p in (fresh, used):
+        s = p.stats()
+        assert s["pipeline_forward"] == 1
+        assert s["launches_forward"] == 2 * math.ceil((wl.nt - 1) / s["time_block"])
+
+
 @pytest.mark.parametrize("nt,K", [(40, 0), (32, 5), (20, 1)])
 @pytest.mark.parametrize("kahan", [True, False])
 @pytest.mark.parametrize("pipeline", [None, 2])

@@ -52,6 +52,77 @@ def rel(a, b):
     return float((a.double() - b.double()).norm() / b.double().norm())
 
 
+def reserved(wl, one_level, call):
+    p = probe_of(wl)
+    if one_level:
+        p.set_option("pipeline", 2)
+        p.set_option("tblock", 1)
+    call(p)                               # kernels loaded, inputs staged
+    p = probe_of(wl)
+    if one_level:
+        p.set_option("pipeline", 2)
+        p.set_option("tblock", 1)
+    before = free()
+    call(p)
+    return before - free(), p.stats()["pipeline_forward"]
+
+
+def test_nonlinear_forward_reserves_no_second_derivative(cuda_device):
+    wl = workload((100, 100), 400, 40, 1)
+    m = torch.tensor(wl.m0, device=cuda_device)
+    out = torch.empty((40, 400, wl.rec.shape[0]), device=cuda_device)
+    resident, route = reserved(wl, False, lambda p: p.forward_nonlinear(m, out=out))
+    assert route == 1
+    assert resident <= reserved(wl, True, lambda p: p.forward_nonlinear(m, out=out))[0] + 16 * MB
+
+
+def test_forward_on_the_one_level_kernels_reserves_no_segments(cuda_device):
+    """A grid that a cluster holds, with so many fields that the one-level kernels are taken."""
+    wl = workload((285, 405), 60, 64, 4)
+    y = torch.tensor(wl.trials, device=cuda_device)
+    out = torch.empty((4, 64, 60, wl.rec.shape[0]), device=cuda_device)
+    got, route = reserved(wl, False, lambda p: p.apply_F(y, out=out))
+    assert route != 1
+    assert got <= reserved(wl, True, lambda p: p.apply_F(y, out=out))[0] + 16 * MB
+
+
+def test_forward_and_migration_in_turn_keep_their_workspace(cuda_device):
+    """A grid on which the Born fields fit a cluster and the adjoint fields do not."""
+    wl = workload((300, 460), 50, 1, 1)
+    p = probe_of(wl)
+    y = torch.tensor(wl.trials, device=cuda_device)
+    d = p.apply_F(y)
+    assert p.stats()["pipeline_forward"] == 1
+    img = p.apply_Fadj(d)
+    assert p.stats()["pipeline_adjoint"] != 1
+    out, im2 = torch.empty_like(d), torch.empty_like(img)
+    left = free()
+    for _ in range(2):
+        p.apply_F(y, out=out)
+        assert free() == left
+        p.apply_Fadj(d, out=im2)
+        assert free() == left
+    assert torch.equal(out, d) and torch.equal(im2, img)
+
+
+@pytest.mark.parametrize("K", [1, 5])
+def test_resident_migration_after_a_one_level_one(cuda_device, K):
+    """The one-level workspace has one segment of Dtt and of injection, the resident kernels take two."""
+    wl = workload((40, 52), 20, 3, 1, pad=4)
+    p = probe_of(wl, ckpt_stride=K)
+    p.set_option("shot_group", 1)
+    d = torch.randn((1, 3, 20, wl.rec.shape[0]), device=cuda_device, generator=torch.Generator(cuda_device).manual_seed(1))
+    ref = p.apply_Fadj(d)
+    assert p.stats()["pipeline_adjoint"] != 1
+    p = probe_of(wl, ckpt_stride=K)
+    p.set_option("autotune", 0)
+    p.apply_Fadj(d)
+    assert p.stats()["pipeline_adjoint"] != 1
+    p.set_option("autotune", 1)
+    assert torch.equal(p.apply_Fadj(d), ref)
+    assert p.stats()["pipeline_adjoint"] == 1
+
+
 @pytest.mark.parametrize("pipeline", [None, 2])
 def test_planned_waves_fit_with_receivers_on_every_row(cuda_device, pipeline):
     """The receiver injection of a segment (200 bands) is most of the workspace."""
