@@ -304,18 +304,37 @@ probe_status encode_ws_maps(probe_t h, WsMaps& m, int R) {
     return PROBE_OK;
 }
 
+// Whether the workspace serves a call as it is.
+bool ws_serves(probe_t h, int W, int nb, int with_ckpt, int with_data, int res) {
+    const Workspace& w = h->ws;
+    const int history = use_history(h, with_ckpt) ? 1 : 0;
+    const int slots = h->ndim == 2 ? dtt_slots_2d(h, with_ckpt, history, res) : 0;
+    // a workspace with checkpoint segments serves calls without them too, in launches of half its planes: calls
+    // with and without in turn keep it
+    const int need = !with_ckpt && w.with_ckpt ? std::min(slots, 2) : slots;
+    const int inj_sets = h->ndim == 2 && with_ckpt && res ? 2 : 1;
+    return w.u && (h->ndim == 3 || w.dtt_slots >= need) && w.inj_sets >= inj_sets && w.W == W && w.nb == nb &&
+           w.with_ckpt >= with_ckpt && w.with_data >= with_data && w.tm_tile_z == h->tile_z && w.history == history;
+}
+
+// Device memory, in bytes, that a call takes besides the workspace that is there (32 MB: 16 arrays in
+// pages of 2 MB).
+double ws_missing(probe_t h, int W, int nb, int with_ckpt, int with_data, int res) {
+    if (ws_serves(h, W, nb, with_ckpt, with_data, res)) return 0.0;
+    return ws_bytes(h, W, nb, with_ckpt, with_data, res).total() - (double)h->ws.bytes + 32e6;
+}
+bool mem_holds(double bytes) {
+    if (bytes <= 0.0) return true;
+    size_t freeb = 0, totb = 0;
+    cudaMemGetInfo(&freeb, &totb);
+    return bytes <= (double)freeb;
+}
+
 probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, int res) {
+    if (ws_serves(h, W, nb, with_ckpt, with_data, res)) return PROBE_OK;
     Workspace& w = h->ws;
     const int G = W;  // image groups for the smallest shot group: any group size fits
     const int history = use_history(h, with_ckpt) ? 1 : 0;
-    const int slots2 = h->ndim == 2 ? dtt_slots_2d(h, with_ckpt, history, res) : 0;
-    // a workspace with checkpoint segments serves calls without them too, in launches of half its planes: calls
-    // with and without in turn keep it
-    const int need = !with_ckpt && w.with_ckpt ? std::min(slots2, 2) : slots2;
-    const int inj_sets = h->ndim == 2 && with_ckpt && res ? 2 : 1;
-    if (w.u && (h->ndim == 3 || w.dtt_slots >= need) && w.inj_sets >= inj_sets && w.W >= W && w.nb >= nb && w.with_ckpt >= with_ckpt && w.with_data >= with_data &&
-        w.groups >= G && w.tm_tile_z == h->tile_z && w.W == W && w.nb == nb && w.history == history)
-        return PROBE_OK;
     free_ws(w);
     auto alloc = [&](void** p, size_t bytes) -> probe_status {
         if (bytes == 0) return PROBE_OK;
@@ -349,8 +368,8 @@ probe_status ensure_ws(probe_t h, int W, int nb, int with_ckpt, int with_data, i
     CK(h, cudaMemset(w.u, 0, s.u));
     CK(h, cudaMemset(w.f, 0, s.f));
     w.history = history;
-    w.inj_sets = inj_sets;
-    w.dtt_slots = h->ndim == 2 ? slots2 : (with_ckpt ? h->K : 2);
+    w.inj_sets = h->ndim == 2 && with_ckpt && res ? 2 : 1;
+    w.dtt_slots = h->ndim == 2 ? dtt_slots_2d(h, with_ckpt, history, res) : (with_ckpt ? h->K : 2);
     if (w.dtt) CK(h, cudaMemset(w.dtt, 0, s.dtt));
     w.W = W;
     w.nb = nb;
@@ -2195,6 +2214,8 @@ probe_status run_op(probe_t h, Op op, const float* dm_dev, const float* data_in,
     if (res_fits(h, need_ckpt, kind == FWD_BORN)) {
         W = plan_wave(h, nbw, need_ckpt, need_data, res_dtt);
         rs = res_set(h, kind, need_ckpt, W, nbw, T);
+        // the one-level kernels need one Dtt segment less: what fits on them alone runs on them
+        if (rs.use && res_dtt && !mem_holds(ws_missing(h, W, nbw, need_ckpt, need_data, 1))) rs = ResSet();
     }
     if (!rs.use) W = plan_wave(h, nbw, need_ckpt, need_data, 0);
     TRY(ensure_ws(h, W, nbw, need_ckpt, need_data, rs.use && res_dtt));
@@ -2545,14 +2566,15 @@ extern "C" probe_status probe_apply_H_group(const probe_t* models, int nmodels, 
     for (int k = 0; k < nmodels; ++k) res = res && res_fits(models[k], 1, 1);
     std::vector<ResSet> rss(nmodels);
     if (res) {  // the resident kernels take the models in turn, the one-level kernels all at once
-        double us = 0.0, fwd = 0.0, rev = 0.0;
+        double us = 0.0, fwd = 0.0, rev = 0.0, missing = 0.0;
         for (int k = 0; k < nmodels; ++k) {
             rss[k] = res_set(models[k], FWD_BORN, true, models[k]->ns, nb[k], h0->K);
             us += rss[k].us;
             fwd += rss[k].fwd;
             rev += rss[k].rev;
+            missing += std::max(0.0, ws_missing(models[k], models[k]->ns, nb[k], 1, 1, 1));
         }
-        res = us < one_level_us(fwd, rev);
+        res = us < one_level_us(fwd, rev) && mem_holds(missing);
     }
     for (int k = 0; k < nmodels; ++k) {
         probe_t h = models[k];

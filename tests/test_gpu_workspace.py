@@ -123,6 +123,36 @@ def test_resident_migration_after_a_one_level_one(cuda_device, K):
     assert p.stats()["pipeline_adjoint"] == 1
 
 
+def test_calls_that_fit_on_the_one_level_kernels_only(cuda_device):
+    """Two Dtt segments of the resident kernels do not fit, one of the one-level kernels does."""
+    from paper_1101_3615_gb300 import apply_H_group
+    wl = workload((100, 100), 401, 64, 1)
+    y = torch.tensor(wl.trials, device=cuda_device)
+
+    def handles():
+        out = [probe_of(wl, ckpt_stride=400) for _ in range(2)]
+        for p in out:
+            p.set_option("shot_wave", 64)     # the caller's wave, not the planner's
+        return out
+
+    probes = handles()
+    ref = probes[0].apply_H(y)
+    assert probes[0].stats()["pipeline_forward"] == 1
+    for o in apply_H_group(probes, [y, y]):
+        assert rel(o, ref) < 1e-6
+    assert probes[0].stats()["pipeline_forward"] == 1
+    probes = handles()
+    with only(3600 * MB):                     # one-level 2.4 GB, resident 4.7 GB
+        for _ in range(2):
+            assert rel(probes[0].apply_H(y), ref) < 1e-6
+        assert probes[0].stats()["pipeline_forward"] != 1
+    with only(4600 * MB):                     # the second model's 2.4 GB fit beside the first's, 4.7 + 4.7 do not
+        for _ in range(2):
+            for o in apply_H_group(probes, [y, y]):
+                assert rel(o, ref) < 1e-6
+        assert probes[0].stats()["pipeline_forward"] != 1
+
+
 @pytest.mark.parametrize("pipeline", [None, 2])
 def test_planned_waves_fit_with_receivers_on_every_row(cuda_device, pipeline):
     """The receiver injection of a segment (200 bands) is most of the workspace."""
