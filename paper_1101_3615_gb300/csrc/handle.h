@@ -71,6 +71,12 @@ struct ResSet {
     ResPlan inc, born, rec, adj;  // incident and Born fields of the forward; recompute and adjoint
 };
 
+// Candidate cluster sizes of a field kind (plan_res2d) with T levels per launch.
+struct ResPlans {
+    int mode = 0, T = 0;
+    std::vector<ResPlan> plans;
+};
+
 struct GraphEntry {
     std::vector<long long> key;
     cudaGraphExec_t exec = nullptr;
@@ -111,9 +117,10 @@ struct probe_s {
     // receivers by pipelined-kernel tile (64 x 16R), R = 1, 2
     int* d_wrec_ptr[3] = {nullptr, nullptr, nullptr};
     int* d_wrec_idx[3] = {nullptr, nullptr, nullptr};
-    int* d_rrec_ptr = nullptr;   // 2D: receivers by grid row (CSR over Nz)
+    int* d_rrec_ptr = nullptr;   // 2D grids that a cluster holds: receivers by grid row (CSR over Nz)
     int* d_rrec_idx = nullptr;
     std::vector<probe::ResSet> res_sets;
+    std::vector<probe::ResPlans> res_plans;
     // 2D adjoint injection: grid rows holding receivers ("bands") and the receiver cells with
     // their receivers (CSR, receiver order), built once per handle
     int* d_rrow = nullptr;       // [Nz] band index or -1

@@ -478,8 +478,10 @@ probe_status build_rec_tiles(probe_t h) {
     TRY(upload_csr(h, key, nkeys, &h->d_rec_tile_ptr, &h->d_rec_tile_idx));
     if (!h->d_rrow) TRY(build_bands(h));
     if (h->ndim == 2) {
-        for (int r = 0; r < h->nr; ++r) key[r] = h->rec_pad[2 * r];  // grid rows (resident kernels)
-        TRY(upload_csr(h, key, h->Nz, &h->d_rrec_ptr, &h->d_rrec_idx));
+        if (res2d_fits(RES_INC, h->kahan != 0, h->Nz, h->Nx, h->pad, 1)) {  // grid rows (resident kernels)
+            for (int r = 0; r < h->nr; ++r) key[r] = h->rec_pad[2 * r];
+            TRY(upload_csr(h, key, h->Nz, &h->d_rrec_ptr, &h->d_rrec_idx));
+        }
         for (int R = 1; R <= 2; ++R) {  // tiles of the pipelined kernels (64 x 16R)
             const int tz = (h->Nz + 16 * R - 1) / (16 * R);
             for (int r = 0; r < h->nr; ++r)
@@ -1145,10 +1147,17 @@ const ResSet& res_set(probe_t h, FwdKind kind, bool adjoint, int W, int nb, int 
     r.key = key;
     const bool born = kind == FWD_BORN, kh = h->kahan != 0;
     if (res_fits(h, adjoint, born)) {
-        const std::vector<ResPlan> inc = plan_res2d(RES_INC, kh, h->Nz, h->Nx, h->pad, T);
+        // (made once per handle, kind and T: they do not depend on the number of fields)
+        auto plans = [&](int mode) {
+            for (const ResPlans& q : h->res_plans)
+                if (q.mode == mode && q.T == T) return q.plans;
+            h->res_plans.push_back({mode, T, plan_res2d(mode, kh, h->Nz, h->Nx, h->pad, T)});
+            return h->res_plans.back().plans;
+        };
+        const std::vector<ResPlan> inc = plans(RES_INC);
         std::vector<ResPlan> bo, ad;
-        if (born) bo = plan_res2d(RES_BORN, kh, h->Nz, h->Nx, h->pad, T);
-        if (adjoint) ad = plan_res2d(RES_ADJ, kh, h->Nz, h->Nx, h->pad, T);
+        if (born) bo = plans(RES_BORN);
+        if (adjoint) ad = plans(RES_ADJ);
         const double seg = 10.0 / T, cells = (double)h->Nz * h->Nx * W * 1e-6;
         r.us = res_pair(inc, W, bo, born ? W * nb : 0, &r.inc, &r.born) + seg;
         r.fwd = cells * (born ? 1 + nb : 1);
