@@ -372,14 +372,20 @@ __global__ void __launch_bounds__(kWsThreads, R == 1 ? 4 : 3) k_fwd2d_ws(const _
 // ---- adjoint ---------------------------------------------------------------
 // Item = (model, shot group, tile); its groups are (shot jj of the group, trial bi of the chunk),
 // jj-major.  s is staged with the item's first group, Dtt with each shot's first trial.
-// Bound: issue slots and load latency together (not DRAM: the levels of 32 shots of 541^2
-// stay in L2).  So the kernel asks for registers that let 4 (one trial) or 3 (two and more) CTAs
-// of one row per thread sit on an SM, instead of 2, and takes the z taps in packed FP32x2.  us per
-// time step, before -> after: 32 shots of 541^2, one trial 43.3 -> 40.9; gradient, 8 shots of 1041^2
-// 37.3 -> 35.3; group of 341^2, 541^2 and 741^2, 8 shots x 4 trials each 158 -> 144.
-// With fewer than three items for each of those CTAs a CTA has too little to pipeline, and the variant
-// of two CTAs per SM stays (MANY = false): Krylov chains on 238 x 584 (9 shots) and 548 x 454 (4 shots)
-// ran 1.2 and 1.1 % slower with four.
+// Bound: issue slots and load latency together while a step's planes stay in L2.  So the kernel asks for
+// registers that let 4 (one trial) or 3 (two and more) CTAs of one row per thread sit on an SM, and takes
+// the z taps in packed FP32x2.  Before, the compiler's own choice let 3 (one trial, 68 registers) or 2 (84 to
+// 94) reside.  us per adjoint step, before -> after: one trial, 541^2, 32 shots in groups of four 43.6 -> 41.0, of
+// one 1041^2, 8 shots, groups of four 37.7 -> 35.6; four trials, 541^2, 16 shots in groups of two 113 -> 86.
+// The variant of two CTAs per SM (MANY = false) stays
+//   * with fewer than three items for each of the CTAs that could reside (launch_adj_nkr).  One trial: 238 x 584,
+//     9 shots in groups of four 11.2 against 11.4 with four, 541^2, 8 shots likewise 15.8 against 16.2; equal
+//     (10.9) on smaller launches.  Several trials would gain with three there too (541^2, 4 shots x 4 trials
+//     41.9 against 32.9);
+//   * with one trial and one shot per image where the step's planes exceed the L2: bound by DRAM, more tiles in flight
+//     then only evict each other's halos.  541^2, 32 and 64 shots 52.5 and 98 against 55.5 and 110 with four,
+//     2841^2, one shot 50.9 against 52.6; just inside the L2 (20 shots, 119 MB) 34.9 against 32.5, equal at
+//     145 MB.  With two shots per image four CTAs stay ahead (64 shots, 303 MB, 80.7 against 75.4).
 constexpr int adj_ctas(int nbc, int r, bool many) { return nbc * r >= 8 ? 1 : r == 2 || !many ? 2 : nbc == 1 ? 4 : 3; }
 
 template <int NBC, bool KAHAN, int S, bool MULTI, int R, bool MANY>
@@ -591,6 +597,16 @@ int num_sms() {
     return n;
 }
 
+double l2_bytes() {
+    static const double n = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, dev);
+        return (double)v;
+    }();
+    return n;
+}
+
 template <typename K>
 cudaError_t launch_persistent(K kernel, size_t smem, int total, const StepParams2D& p, cudaStream_t st) {
     static_assert(sizeof(StepParams2D) < 32000, "kernel parameter block too large");
@@ -632,8 +648,16 @@ cudaError_t launch_adj_nkrm(int stages, const StepParams2D& q, cudaStream_t st) 
 template <int NB, bool KH, int R>
 cudaError_t launch_adj_nkr(int stages, const StepParams2D& q, cudaStream_t st) {
     constexpr int ctas = adj_ctas(NB, R, true);
-    if constexpr (ctas > 2)
-        if (q.total_items >= 3 * num_sms() * ctas) return launch_adj_nkrm<NB, KH, R, true>(stages, q, st);
+    if constexpr (ctas > 2) {
+        double planes = 0.0;  // bytes of the step: three field levels, Dtt, image and compensation
+        bool single = NB == 1;
+        for (int k = 0; k < q.nmodels; ++k) {
+            planes += 4.0 * q.m[k].F * (3.0 * q.m[k].nshots + 2.0 * q.m[k].ngroups);
+            single = single && q.m[k].shot_group == 1;
+        }
+        if (q.total_items >= 3 * num_sms() * ctas && !(single && planes > 1.125 * l2_bytes()))
+            return launch_adj_nkrm<NB, KH, R, true>(stages, q, st);
+    }
     return launch_adj_nkrm<NB, KH, R, false>(stages, q, st);
 }
 

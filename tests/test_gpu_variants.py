@@ -66,12 +66,12 @@ def test_autotuned_group_on_the_one_level_kernels(cuda_device):
         assert rel(a, probe_of(w, pipeline=0, shot_group=1).apply_H(d)) < 1e-6   # the order of the image sums
 
 
-@pytest.mark.parametrize("nb", [1, 3])
-def test_adjoint_with_many_items_gives_identical_bits(cuda_device, nb):
+@pytest.mark.parametrize("ns,nb", [(6, 1), (6, 3), (32, 1)])
+def test_adjoint_with_many_items_gives_identical_bits(cuda_device, ns, nb):
     """Six shots of 306 tiles: more than three items for each of four (three) CTAs per SM of 152 SMs, by
-    itself and in a group of two models of three shots."""
+    itself and in a group of two models of half the shots; 32 shots: planes beyond the L2."""
     from paper_1101_3615_gb300 import apply_H_group
-    wl, half = workload((531, 531), 20, 6, nb), workload((531, 531), 20, 3, nb)
+    wl, half = workload((531, 531), 20, ns, nb), workload((531, 531), 20, ns // 2, nb)
     y = torch.tensor(wl.trials, device=cuda_device)
     for S in (2, 3):
         one, many = probe_of(wl, pipeline=0, shot_group=1), probe_of(wl, pipeline=S, pipe_rows=1, shot_group=1)
