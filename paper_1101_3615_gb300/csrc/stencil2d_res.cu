@@ -16,7 +16,7 @@
 // are bound by launch and first-load latency on such grids.  Measured, whole calls, one-level kernels ->
 // here: F on 77 x 103, 1 shot, 3 trials, nt = 200 1.79 -> 0.366 ms; H on 141 x 141, 4 shots, nt = 800 12.8 ->
 // 2.77 ms; four H in a chain on 241 x 281, 6 shots, nt = 400 38.2 -> 11.0 ms; F* on 277 x 423, 12 shots,
-// 2 data sets, nt = 700 29.1 -> 15.7 ms.
+// 2 data sets, nt = 700 29.1 -> 15.6 ms.
 //
 // The two halves of the halo exchange need no second barrier: the rows whose update reads a
 // neighbour's halo rows are exactly the rows sent to that neighbour, so the arrival of all their
@@ -414,7 +414,8 @@ bool res2d_fits(int mode, bool kahan, int Nz, int Nx, int pad, int nsteps) {
 }
 
 // Candidate cluster sizes (not only powers of two: with 9 CTAs the chip holds 15 clusters, as with 8,
-// and a strip is an eighth lower; 241 x 281, 6 shots, Krylov trials 13.4 -> 11.1 ms) and rows per
+// and a strip is an eighth lower; 241 x 281, 6 shots, Krylov trials 13.4 -> 11.1 ms; 11, 13 and 15 have
+// not been timed) and rows per
 // thread for fields of an Nz x Nx grid, each with the number of
 // clusters that the chip holds at once and the estimated time of one level of one wave of clusters.
 // The model (microseconds), fitted on 77 x 103 to 277 x 423 grids, C = 1 to 16, within about 15 %:

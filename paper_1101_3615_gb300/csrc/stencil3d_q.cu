@@ -18,7 +18,8 @@
 // the incident step (168 x 256 x 296, 4 shots, 4 trials).  Measured against the kernels of
 // stencil3d.cu as they were tuned, whole calls: H on 296^3 (padded), 8 shots, 4 trials, 60 levels 528 ->
 // 465 ms; H on 116 x 101 x 141, 3 shots 45.2 -> 34.7 ms; F on 168^3, 4 shots, 2 trials 42.9 -> 38.8 ms.
-// Slower variants: two trials per CTA, two rows per thread, a refill by the last compute warp.
+// Slower variants: two trials per CTA, two rows per thread, a refill by the last compute warp.  At the 96
+// registers that two CTAs per SM leave, every instantiation spills (16 to 84 bytes stored per thread).
 //
 // The per-cell arithmetic is that of cells3 in stencil3d.cu, operation for operation: same bits.
 #include "common.cuh"
