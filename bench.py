@@ -110,8 +110,6 @@ def profile_run(a, wl):
     dev = torch.device("cuda", 0)
     p = Probe(wl.m0, wl.h, wl.dt, wl.nt, wl.pad, wl.src, wl.rec, wl.wavelet, snapshot_dtype=a.snapshot)
     p.set_option("check_finite", 0)
-    if len(wl.shape) == 2:
-        p.set_option("tile_z", 16)
     if a.pipeline >= 0:               # fixed kernel variant (no timing under the profiler)
         p.set_option("pipeline", a.pipeline)
         if a.pipe_rows:
@@ -497,7 +495,6 @@ def _probe(wl, **kw):
     p = Probe(wl.m0, wl.h, wl.dt, wl.nt, wl.pad, wl.src, wl.rec, wl.wavelet, **kw)
     p.set_option("check_finite", 0)
     if len(wl.shape) == 2:
-        p.set_option("tile_z", 16)
         p.set_option("use_graph", 1)
     return p
 
@@ -798,7 +795,6 @@ def main():
     p.set_option("check_finite", 0)
     is3d = len(wl.shape) == 3
     if not is3d:
-        p.set_option("tile_z", 16)
         p.set_option("use_graph", 1)  # each shot wave's sweeps replayed as one CUDA graph
     if a.fixed:
         pf, pa, rows, grp = (int(v) for v in a.fixed.split(","))
