@@ -109,7 +109,7 @@ typedef enum {
     PROBE_OPT_SHOT_WAVE = 2,     /* max shots resident at once; 0 (default) = memory planner */
     PROBE_OPT_SHOT_GROUP = 3,    /* 2D: shots per CTA in the adjoint sweep; 3D: shots per adjoint cluster
                                     (PROBE_OPT_CLUSTER3D bit 1); 0 = autotuned (2D) or 4 (3D) */
-    PROBE_OPT_USE_GRAPH = 4,     /* 1 (default): replay sweeps from a captured CUDA graph */
+    PROBE_OPT_USE_GRAPH = 4,     /* 1: replay 2D sweeps from a captured CUDA graph; 0 (default): launch them */
     PROBE_OPT_TIMING = 5,        /* CUDA-event timings read by probe_get_stats (recorded on the call's
                                     stream, also inside replayed graphs; no call synchronises):
                                     1 = every sweep (forward, recompute, adjoint), 2 = the forward
